@@ -47,22 +47,12 @@
 #include "mhr_internal.cuh"
 #include "mhr_query.cuh"
 #include "mhr_mlp_tc.cuh"
+#include "mhr_score.cuh"
 #include "mhr_util.cuh"
 
 namespace mhr {
 
 constexpr unsigned FULL = 0xffffffffu;
-
-__device__ __forceinline__ int64_t upper_bound_i64(const int64_t* __restrict__ a, int64_t n, int64_t x) {
-    // first index i in [0, n) with a[i] > x (n if none)
-    int64_t lo = 0, hi = n;
-    while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
-        if (a[mid] <= x) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
 
 __device__ __forceinline__ unsigned lanemask_lt() {
     unsigned m;
@@ -298,8 +288,6 @@ __device__ __forceinline__ void slot_commit(const PlanDev* __restrict__ P, const
 // parallel; then groups of G lanes score the 32 edges, H = 32 / G at a time.
 __global__ void __launch_bounds__(256) k_expand(const PlanDev* __restrict__ P, DevGraph g) {
     const int lane = threadIdx.x & 31;
-    const int G = P->score_width, H = 32 / G;
-    const int sub = lane & (G - 1);
     const int64_t X = P->X;
     const int64_t warp_id = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
     const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -307,56 +295,10 @@ __global__ void __launch_bounds__(256) k_expand(const PlanDev* __restrict__ P, D
         const int64_t x = base + lane;
         const bool live = x < X;
         const SlotInfo o = slot_info(P, g, x, live);
-        const uint32_t hu = o.sideA ? o.s : o.vtx, tv = o.sideA ? o.vtx : o.t;
-        float wmine = 0.f;
-        for (int rd = 0; rd < G; ++rd) {
-            const int src = rd * H + lane / G;
-            const uint32_t a = __shfl_sync(0xffffffffu, hu, src);
-            const uint32_t rr = __shfl_sync(0xffffffffu, o.r, src);
-            const uint32_t b = __shfl_sync(0xffffffffu, tv, src);
-            // dead lanes score vertex 0's rows
-            const float w = edge_w32_group(g, a, rr, b, sub, G);
-            const float tw = __shfl_sync(0xffffffffu, w, ((lane - rd * H) & (H - 1)) * G);
-            if (lane / H == rd) wmine = tw;
-        }
-        slot_commit(P, g, x, live, o, wmine, lane);
+        // dead lanes score vertex 0's rows
+        const float w = warp_score_any(g, o.sideA ? o.s : o.vtx, o.r, o.sideA ? o.vtx : o.t, P->score_width, lane);
+        slot_commit(P, g, x, live, o, w, lane);
     }
-}
-
-// Query of a slot at position lx of one side: the last q with offs[q] <= lx.
-// The warp's live slots are consecutive and on one side, so the warp finds
-// the query q0 of its first slot (position lx0) with a 32-ary search (three
-// rounds of one load per lane for 4,096 queries instead of twelve dependent
-// loads per lane), then each lane counts the query starts after q0 that are
-// <= lx among the next 32 (five shuffle steps).  A lane with more than 31
-// query starts between lx0 and lx (empty queries) searches on its own.
-__device__ __forceinline__ int warp_query_of(const int64_t* __restrict__ offs, int nq, int64_t lx0, int64_t lx,
-                                             int lane) {
-    int64_t lo = 0, span = static_cast<int64_t>(nq) + 1;  // offs[lo] <= lx0 < offs[lo + span] (or the end)
-    while (span > 32) {
-        const int64_t step = (span + 31) >> 5;
-        const int64_t j = lane * step;
-        const bool le = j < span && offs[lo + j] <= lx0;
-        const int64_t c = __popc(__ballot_sync(0xffffffffu, le));  // >= 1: offs[lo] <= lx0
-        const int64_t nlo = (c - 1) * step;
-        span = min(step, span - nlo);
-        lo += nlo;
-    }
-    {
-        const bool le = lane < span && offs[lo + lane] <= lx0;
-        lo += __popc(__ballot_sync(0xffffffffu, le)) - 1;
-    }
-    const int64_t j = lo + 1 + lane;
-    const int64_t b = j <= nq ? offs[j] : INT64_MAX;
-    int own = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-        const int64_t pv = __shfl_sync(0xffffffffu, b, own + step - 1);
-        if (pv <= lx) own += step;
-    }
-    const int64_t b31 = __shfl_sync(0xffffffffu, b, 31);
-    if (b31 <= lx) return static_cast<int>(upper_bound_i64(offs, nq + 1, lx) - 1);
-    return static_cast<int>(lo) + own;
 }
 
 // slot_info without the scan degree, the query found warp-cooperatively.
@@ -377,9 +319,12 @@ __device__ __forceinline__ SlotInfo slot_locate_warp(const PlanDev* __restrict__
     const int64_t lx = live ? (sA ? x : x - totA) : 0;
     int q = 0;
     if (uniform) {
+        // the warp's live slots are consecutive and on one side: one search for
+        // the first slot's query, then each lane's among the next starts
         const int64_t* offs = mC == 0u ? P->a_off : P->c_off;
         const int64_t lx0 = __shfl_sync(0xffffffffu, lx, 0);
-        q = warp_query_of(offs, P->nq, lx0, live ? lx : lx0, lane);
+        const int64_t q0 = warp_row_search(offs, P->nq, lx0, lane);
+        q = static_cast<int>(warp_rows_from(offs, P->nq, q0, live ? lx : lx0, lane));
     } else if (live) {
         q = static_cast<int>(upper_bound_i64(sA ? P->a_off : P->c_off, P->nq + 1, lx) - 1);
     }
@@ -405,125 +350,27 @@ __device__ __forceinline__ SlotInfo slot_locate_warp(const PlanDev* __restrict__
 }
 
 // k_expand for rows of at most two 16-byte vectors per lane of a G-lane group
-// (bf16 with d % 8 == 0 and d / 8 <= 2G, fp32 with d % 4 == 0 and d / 4 <=
-// 2G).  The rows of the random side (the slot's far endpoint) of up to four
-// rounds are loaded before any arithmetic, with the endpoint's scan-degree
-// loads beside them, so a warp keeps up to four rows per group in flight
-// instead of one; the fixed side (the query's s or t) and the relation row
-// are the same few rows for many slots and come from L1.  The group sums of
-// RB rounds are reduced together: plain xor steps down to RB lanes, then a
-// butterfly in which each step halves the rounds a lane carries, so lane
-// `sub` ends with round (sub mod RB): RB - 1 shuffles for the last log2(RB)
-// steps of RB rounds instead of RB log2(RB).  Every lane still adds its own partial to
-// its partner's at each step of the same xor tree, and fp32 addition is
-// commutative, so with the same per-element expression and the same order
-// within a lane the weights are those edge_w32_group computes.
-// Four rounds at a time and three 256-thread blocks per SM (80 registers)
-// measured fastest on the batching workload (3.31 ms per launch; eight rounds
-// at two blocks per SM 3.88 ms; two rounds at four blocks 3.32 ms).
-constexpr int kExpandRounds = 4;
+// (warp_score_v); the endpoint's scan-degree loads are issued beside its row's.
 template <int G>
 __global__ void __launch_bounds__(256, 3) k_expand_v(const PlanDev* __restrict__ P, DevGraph g) {
-    constexpr int H = 32 / G;
-    constexpr int RB = G < kExpandRounds ? G : kExpandRounds;  // rounds loaded and reduced together
-    const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const int sub = lane & (G - 1);
     const int64_t X = P->X;
     const int64_t warp_id = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
     const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    const bool f32 = g.dtype == MHR_F32;
-    const bool transe = g.fn == MHR_SCORE_TRANSE_L1;
-    const int nvec = f32 ? (g.d >> 2) : (g.d >> 3);  // 16-byte vectors per row
-    const bool h0 = sub < nvec, h1 = sub + G < nvec;
-    const uint4* E = static_cast<const uint4*>(g.vemb);
-    const uint4* Rw = static_cast<const uint4*>(g.remb);
-    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
     for (int64_t base = warp_id * 32; base < X; base += nwarps * 32) {  // warp-uniform
         const int64_t x = base + lane;
         const bool live = x < X;
         SlotInfo o = slot_locate_warp(P, g, x, live, lane);
-        const uint32_t fixv = o.sideA ? o.s : o.t;               // dead lanes: vertex 0
-        const uint32_t rsa = (o.r << 1) | (o.sideA ? 1u : 0u);   // relation and side, one shuffle
         const int64_t* so = o.sideA ? g.off : g.roff;
         int64_t d0 = 0, d1 = 0;
         if (live) {
             d0 = so[o.vtx];
             d1 = so[o.vtx + 1];
         }
-        float wmine = 0.f;
-#pragma unroll
-        for (int rb = 0; rb < G; rb += RB) {
-            uint4 C0[RB], C1[RB];
-#pragma unroll
-            for (int i = 0; i < RB; ++i) {
-                const int src = (rb + i) * H + lane / G;
-                const int64_t v = __shfl_sync(FULL, o.vtx, src);
-                C0[i] = h0 ? __ldg(E + v * nvec + sub) : z;
-                C1[i] = h1 ? __ldg(E + v * nvec + sub + G) : z;
-            }
-            float acc[RB];
-#pragma unroll
-            for (int i = 0; i < RB; ++i) {
-                const int src = (rb + i) * H + lane / G;
-                const uint32_t q2 = __shfl_sync(FULL, rsa, src);
-                const int64_t rr = q2 >> 1;
-                const bool sa = (q2 & 1u) != 0u;
-                const int64_t fv = __shfl_sync(FULL, fixv, src);
-                const uint4 F0 = h0 ? __ldg(E + fv * nvec + sub) : z, B0 = h0 ? __ldg(Rw + rr * nvec + sub) : z;
-                const uint4 F1 = h1 ? __ldg(E + fv * nvec + sub + G) : z,
-                            B1 = h1 ? __ldg(Rw + rr * nvec + sub + G) : z;
-                // side A: the edge (s, r, vtx), head fixed; side C: (vtx, r, t), tail fixed
-                const uint4 As[2] = {sa ? F0 : C0[i], sa ? F1 : C1[i]};
-                const uint4 Cs[2] = {sa ? C0[i] : F0, sa ? C1[i] : F1};
-                const uint4 Bs[2] = {B0, B1};
-                float a_ = 0.f;
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    if (k == 0 && !h0) break;
-                    if (k == 1 && !h1) break;
-                    const uint32_t a[4] = {As[k].x, As[k].y, As[k].z, As[k].w};
-                    const uint32_t b[4] = {Bs[k].x, Bs[k].y, Bs[k].z, Bs[k].w};
-                    const uint32_t c[4] = {Cs[k].x, Cs[k].y, Cs[k].z, Cs[k].w};
-                    if (f32) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            a_ += term_tr(__uint_as_float(a[e]), __uint_as_float(b[e]), __uint_as_float(c[e]), transe);
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            a_ += term_tr(bf_lo(a[e]), bf_lo(b[e]), bf_lo(c[e]), transe);
-                            a_ += term_tr(bf_hi(a[e]), bf_hi(b[e]), bf_hi(c[e]), transe);
-                        }
-                    }
-                }
-                acc[i] = a_;
-            }
-            // xor steps G/2 .. RB: every round's sum over lanes that differ in those bits
-#pragma unroll
-            for (int off = G >> 1; off >= RB; off >>= 1)
-#pragma unroll
-                for (int i = 0; i < RB; ++i) acc[i] += __shfl_xor_sync(FULL, acc[i], off, G);
-            // butterfly over the low log2(RB) bits: keep the half of the rounds
-            // selected by this lane's bit, send the other half to the partner
-#pragma unroll
-            for (int off = RB >> 1; off > 0; off >>= 1) {
-                const bool hi = (sub & off) != 0;
-#pragma unroll
-                for (int j = 0; j < off; ++j) {
-                    const float send = hi ? acc[j] : acc[j + off];
-                    const float keep = hi ? acc[j + off] : acc[j];
-                    acc[j] = keep + __shfl_xor_sync(FULL, send, off, G);
-                }
-            }
-            // lane sub of group gi now holds round rb + (sub mod RB) of slot (round) * H + gi
-            const float w = transe ? __fsub_rn(g.gamma32, acc[0]) : acc[0];
-            const int rd = lane / H;
-            const float tw = __shfl_sync(FULL, w, (lane & (H - 1)) * G + (rd & (RB - 1)));
-            if (rd >= rb && rd < rb + RB) wmine = tw;
-        }
+        // side A: the edge (s, r, vtx), head fixed; side C: (vtx, r, t), tail fixed; dead lanes: vertex 0
+        const float w = warp_score_v<G>(g, o.sideA ? o.s : o.t, o.vtx, (o.r << 1) | (o.sideA ? 1u : 0u), lane);
         o.sdeg = static_cast<uint32_t>(d1 - d0);
-        slot_commit(P, g, x, live, o, wmine, lane);
+        slot_commit(P, g, x, live, o, w, lane);
     }
 }
 
@@ -531,9 +378,7 @@ using ExpandKernel = void (*)(const PlanDev*, DevGraph);
 
 // the expansion kernel for a graph's rows and group width
 static ExpandKernel expand_kernel(const DevGraph& g, int G) {
-    const bool vec2 = g.dtype == MHR_F32 ? ((g.d & 3) == 0 && (g.d >> 2) <= 2 * G)
-                                         : ((g.d & 7) == 0 && (g.d >> 3) <= 2 * G);
-    if (!vec2) return k_expand;
+    if (!score_vec2(g, G)) return k_expand;
     switch (G) {
         case 1: return k_expand_v<1>;
         case 2: return k_expand_v<2>;
@@ -2880,15 +2725,6 @@ static cudaError_t launch_graphs(Plan* p, cudaStream_t st) {
         if ((e = cudaGraphLaunch(p->exec[part], st)) != cudaSuccess) return e;
     }
     return cudaEventRecord(p->ev[3], st);
-}
-
-// lanes that score one edge together: about `per` 16-byte vectors per lane per row
-static int hit_group_width(int d, int dtype, int per) {
-    const int vec = (dtype == MHR_F32) ? ((d & 3) == 0 ? d / 4 : d) : ((d & 7) == 0 ? d / 8 : d);
-    const int want = (vec + per - 1) / per;
-    int w = 1;
-    while (w < want && w < 32) w <<= 1;
-    return w;
 }
 
 static float __double2float_ru_host(double x) {

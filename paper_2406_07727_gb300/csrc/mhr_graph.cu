@@ -15,6 +15,7 @@
 
 #include "mhr_internal.cuh"
 #include "mhr_score.cuh"
+#include "mhr_sort.cuh"
 #include "mhr_util.cuh"
 #include <cuda_bf16.h>
 
@@ -78,25 +79,35 @@ __global__ void k_validate_offsets(const int64_t* __restrict__ off, int64_t n, i
     if (blockIdx.x == 0 && threadIdx.x == 0 && (off[0] != 0 || off[n] != E)) err[kErrOffsets] = 1;
 }
 
-__global__ void k_validate_rows(const int64_t* __restrict__ off, const uint32_t* __restrict__ col,
-                                const uint16_t* __restrict__ rel, int64_t n, int32_t R,
-                                int* __restrict__ err) {
+// Checks every edge and writes its source.  Each warp walks consecutive edges
+// (the rows of the next 32 are found among the row starts after the last one),
+// so short and empty rows cost what long ones do: 20 M edges in 0.1 ms (a warp
+// per row took 1.26 ms).
+__global__ void k_validate_edges(const int64_t* __restrict__ off, const uint32_t* __restrict__ col,
+                                 const uint16_t* __restrict__ rel, int64_t n, int64_t E, int32_t R,
+                                 uint32_t* __restrict__ src, int* __restrict__ err) {
     const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
+    const int64_t warp_id = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
     const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    for (int64_t u = warp; u < n; u += nwarps) {
-        const int64_t lo = off[u], hi = off[u + 1];
-        for (int64_t p = lo + lane; p < hi; p += 32) {
-            const uint32_t c = col[p];
-            const uint32_t r = rel[p];
-            if (c >= static_cast<uint64_t>(n)) err[kErrColRange] = 1;
-            if (r >= static_cast<uint32_t>(R)) err[kErrRelRange] = 1;
-            if (c == static_cast<uint64_t>(u)) err[kErrSelfLoop] = 1;
-            if (p > lo) {
-                const uint32_t pc = col[p - 1];
-                const uint32_t pr = rel[p - 1];
-                if (!(pc < c || (pc == c && pr < r))) err[kErrRowOrder] = 1;
-            }
+    const int64_t steps = (E + 31) >> 5;
+    const int64_t s0 = steps * warp_id / nwarps, s1 = steps * (warp_id + 1) / nwarps;
+    if (s0 >= s1) return;  // warp-uniform
+    int64_t row = warp_row_search(off, n, s0 * 32, lane);
+    for (int64_t st = s0; st < s1; ++st) {
+        const int64_t p = st * 32 + lane;
+        const int64_t u = warp_rows_from(off, n, row, min(p, E - 1), lane);
+        row = __shfl_sync(0xffffffffu, u, 31);
+        if (p >= E) continue;
+        const uint32_t c = col[p];
+        const uint32_t r = rel[p];
+        src[p] = static_cast<uint32_t>(u);
+        if (c >= static_cast<uint64_t>(n)) err[kErrColRange] = 1;
+        if (r >= static_cast<uint32_t>(R)) err[kErrRelRange] = 1;
+        if (c == static_cast<uint64_t>(u)) err[kErrSelfLoop] = 1;
+        if (p > off[u]) {
+            const uint32_t pc = col[p - 1];
+            const uint32_t pr = rel[p - 1];
+            if (!(pc < c || (pc == c && pr < r))) err[kErrRowOrder] = 1;
         }
     }
 }
@@ -120,14 +131,6 @@ __global__ void k_count_in(const uint32_t* __restrict__ col, int64_t E, uint32_t
         atomicAdd(&indeg[col[p]], 1u);
 }
 
-__global__ void k_make_keys(const uint32_t* __restrict__ col, int64_t E, int64_t N,
-                            uint64_t* __restrict__ keys) {
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t p = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; p < N; p += stride)
-        keys[p] = p < E ? ((static_cast<uint64_t>(col[p]) << 32) | static_cast<uint64_t>(p))
-                        : ~0ull;
-}
-
 __device__ __forceinline__ int64_t row_of_edge(const int64_t* __restrict__ off, int64_t n, int64_t p) {
     // largest u with off[u] <= p (rows may be empty)
     int64_t lo = 0, hi = n;  // answer in [0, n)
@@ -139,14 +142,15 @@ __device__ __forceinline__ int64_t row_of_edge(const int64_t* __restrict__ off, 
     return lo;
 }
 
-__global__ void k_fill_reverse(const uint64_t* __restrict__ keys, int64_t E,
-                               const int64_t* __restrict__ off, int64_t n,
+// edge[i]: the CSR edges sorted by destination (stable, so a row is in
+// (source, relation) order)
+__global__ void k_fill_reverse(const uint32_t* __restrict__ edge, int64_t E, const uint32_t* __restrict__ src,
                                const uint16_t* __restrict__ rel, uint32_t* __restrict__ rcol,
                                uint16_t* __restrict__ rrel) {
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < E; i += stride) {
-        const int64_t p = static_cast<int64_t>(keys[i] & 0xffffffffull);
-        rcol[i] = static_cast<uint32_t>(row_of_edge(off, n, p));
+        const uint32_t p = edge[i];
+        rcol[i] = src[p];
         rrel[i] = rel[p];
     }
 }
@@ -154,41 +158,46 @@ __global__ void k_fill_reverse(const uint64_t* __restrict__ keys, int64_t E,
 // ---------------------------------------------------------------------------
 // norms behind the fp32 error bound
 // ---------------------------------------------------------------------------
-__global__ void k_row_norms(const void* __restrict__ tab, int dtype, int64_t rows, int d,
-                            unsigned long long* __restrict__ max_l1,
-                            unsigned long long* __restrict__ max_aux, int aux_is_inf) {
-    // max over rows of ||x||_1 and of ||x||_2^2 (or ||x||_inf); non-negative
-    // doubles compare like their bit patterns, so atomicMax on the bits works.
-    __shared__ double s1[32], s2[32];
-    double m1 = 0.0, m2 = 0.0;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t r = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; r < rows; r += stride) {
-        double l1 = 0.0, aux = 0.0;
-        for (int j = 0; j < d; ++j) {
-            double x = fabs(static_cast<double>(emb_f32(tab, dtype, r, d, j)));
-            l1 += x;
-            aux = aux_is_inf ? fmax(aux, x) : aux + x * x;
-        }
-        m1 = fmax(m1, l1);
-        m2 = fmax(m2, aux);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        m1 = fmax(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-        m2 = fmax(m2, __shfl_xor_sync(0xffffffffu, m2, o));
-    }
+// Upper bounds of the largest ||x||_1 and of the largest ||x||_2^2 (or
+// ||x||_inf) over the rows: a warp per row, fp32 sums rounded up at every step
+// (at most d * 2^-23 above the exact norm, in the safe direction).  Sums in fp64
+// by one thread per row were bound by the fp64 pipe and by uncoalesced loads:
+// 1.0 ms for 1 M rows of 128 fp32 values.
+__global__ void __launch_bounds__(256) k_row_norms(const void* __restrict__ tab, int dtype, int64_t rows, int d,
+                                                   unsigned long long* __restrict__ max_l1,
+                                                   unsigned long long* __restrict__ max_aux, int aux_is_inf) {
+    __shared__ float s1[8], s2[8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    float m1 = 0.f, m2 = 0.f;
+    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+    for (int64_t r = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5; r < rows; r += nwarps) {
+        float l1 = 0.f, aux = 0.f;
+        for (int j = lane; j < d; j += 32) {
+            const float x = fabsf(emb_f32(tab, dtype, r, d, j));
+            l1 = __fadd_ru(l1, x);
+            aux = aux_is_inf ? fmaxf(aux, x) : __fadd_ru(aux, __fmul_ru(x, x));
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            l1 = __fadd_ru(l1, __shfl_xor_sync(0xffffffffu, l1, o));
+            const float y = __shfl_xor_sync(0xffffffffu, aux, o);
+            aux = aux_is_inf ? fmaxf(aux, y) : __fadd_ru(aux, y);
+        }
+        m1 = fmaxf(m1, l1);
+        m2 = fmaxf(m2, aux);
+    }
     if (lane == 0) {
         s1[wid] = m1;
         s2[wid] = m2;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-            m1 = fmax(m1, s1[w]);
-            m2 = fmax(m2, s2[w]);
+        for (int w = 1; w < static_cast<int>(blockDim.x >> 5); ++w) {
+            m1 = fmaxf(m1, s1[w]);
+            m2 = fmaxf(m2, s2[w]);
         }
-        atomicMax(max_l1, static_cast<unsigned long long>(__double_as_longlong(m1)));
-        atomicMax(max_aux, static_cast<unsigned long long>(__double_as_longlong(m2)));
+        // non-negative doubles compare like their bit patterns
+        atomicMax(max_l1, static_cast<unsigned long long>(__double_as_longlong(static_cast<double>(m1))));
+        atomicMax(max_aux, static_cast<unsigned long long>(__double_as_longlong(static_cast<double>(m2))));
     }
 }
 
@@ -469,7 +478,29 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
     MHR_CUDA_TRY(cudaStreamSynchronize(st));
     if (herr[kErrOffsets])
         return fail(MHR_EINVAL, "offsets must start at 0, be non-decreasing and end at n_edges");
-    k_validate_rows<<<grid, 256, 0, st>>>(off, col, rel, n, R, err);
+    // scratch of the reverse sort, and the source of every edge
+    uint32_t* src = nullptr;
+    SortScratch ss{};
+    if (E) {
+        const size_t tiles = sort_tiles(static_cast<uint64_t>(E)), nc = 256 * tiles;
+        const size_t eb = (sizeof(uint32_t) * E + 255) / 256 * 256, cb = (sizeof(int64_t) * (nc + 1) + 255) / 256 * 256;
+        char* mem;
+        MHR_CUDA_TRY(tmp.alloc(&mem, 5 * eb + 2 * cb + 256 + sizeof(int64_t) * kScanPartials));
+        src = reinterpret_cast<uint32_t*>(mem);
+        for (int i = 0; i < 2; ++i) {
+            ss.key[i] = reinterpret_cast<uint32_t*>(mem + (1 + i) * eb);
+            ss.val[i] = reinterpret_cast<uint32_t*>(mem + (3 + i) * eb);
+        }
+        mem += 5 * eb;
+        ss.counts = reinterpret_cast<uint32_t*>(mem);
+        ss.offsets = reinterpret_cast<int64_t*>(mem + cb);
+        ss.n_counts = reinterpret_cast<int64_t*>(mem + 2 * cb);
+        ss.partials = reinterpret_cast<int64_t*>(mem + 2 * cb + 256);
+        const int64_t nch = static_cast<int64_t>(nc);
+        MHR_CUDA_TRY(cudaMemcpyAsync(ss.n_counts, &nch, sizeof nch, cudaMemcpyHostToDevice, st));
+        MHR_CUDA_TRY(cudaMemsetAsync(ss.partials, 0, sizeof(int64_t) * kScanPartials, st));
+        k_validate_edges<<<grid, 256, 0, st>>>(off, col, rel, n, E, R, src, err);
+    }
     k_validate_finite<<<grid, 256, 0, st>>>(vemb, desc->emb_dtype, n * d, err);
     k_validate_finite<<<grid, 256, 0, st>>>(remb, desc->emb_dtype, static_cast<int64_t>(R) * d, err);
     MHR_CUDA_TRY(cudaGetLastError());
@@ -501,13 +532,11 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
         if (E) k_count_in<<<grid, 256, 0, st>>>(col, E, indeg);
         MHR_CUDA_TRY(device_excl_scan<uint32_t>(indeg, n_dev, partials, roff, st));
         if (E) {
-            int64_t N = kBitonicTile;
-            while (N < E) N <<= 1;
-            uint64_t* keys;
-            MHR_CUDA_TRY(tmp.alloc(&keys, sizeof(uint64_t) * N));
-            k_make_keys<<<grid, 256, 0, st>>>(col, E, N, keys);
-            MHR_CUDA_TRY(bitonic_sort_u64(keys, static_cast<uint64_t>(N), std::max(1, g->num_sms), st));
-            k_fill_reverse<<<grid, 256, 0, st>>>(keys, E, off, n, rel, rcol, rrel);
+            int bits = 1;
+            while (((n - 1) >> bits) != 0) ++bits;
+            uint32_t* edge;
+            MHR_CUDA_TRY(radix_sort_pairs(col, nullptr, static_cast<uint32_t>(E), bits, ss, &edge, st));
+            k_fill_reverse<<<grid, 256, 0, st>>>(edge, E, src, rel, rcol, rrel);
             MHR_CUDA_TRY(cudaGetLastError());
         }
         // the scan wrote n_dev-long output plus the total at roff[n]
@@ -525,7 +554,7 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
     MHR_CUDA_TRY(tmp.alloc(&mx, sizeof(unsigned long long) * 4));
     MHR_CUDA_TRY(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * 4, st));
     k_row_norms<<<grid, 256, 0, st>>>(vemb, desc->emb_dtype, n, d, mx + 0, mx + 1, 0);
-    k_row_norms<<<std::max(1, std::min(grid, (R + 255) / 256)), 256, 0, st>>>(remb, desc->emb_dtype, R, d,
+    k_row_norms<<<std::max(1, std::min(grid, (R + 7) / 8)), 256, 0, st>>>(remb, desc->emb_dtype, R, d,
                                                                                mx + 2, mx + 3, 1);
     MHR_CUDA_TRY(cudaGetLastError());
     unsigned long long hm[4];

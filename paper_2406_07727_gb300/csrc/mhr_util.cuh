@@ -1,7 +1,6 @@
 // Device-wide building blocks: block scans, a fixed-grid exclusive scan whose
 // length is read from device memory (so it can live inside a captured CUDA
-// graph while the length changes between replays), and a bitonic sort of
-// 64-bit keys used once per graph load.
+// graph while the length changes between replays).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -122,66 +121,6 @@ inline cudaError_t device_excl_scan(const TIn* in, const int64_t* n_dev, int64_t
                                     int64_t* out, cudaStream_t st) {
     scan_partials_kernel<TIn><<<kScanGrid, kScanThreads, 0, st>>>(in, n_dev, partials);
     scan_apply_kernel<TIn><<<kScanGrid, kScanThreads, 0, st>>>(in, n_dev, partials, out);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// Bitonic sort of N = 2^k uint64 keys, ascending.  Stages with stride below
-// kBitonicTile/2 run inside shared memory.
-// ---------------------------------------------------------------------------
-constexpr int kBitonicThreads = 1024;
-constexpr int kBitonicTile = 2 * kBitonicThreads;
-
-static __global__ void __launch_bounds__(kBitonicThreads)
-bitonic_shared_kernel(uint64_t* __restrict__ keys, uint64_t kmin, uint64_t kmax_stage) {
-    // runs stages (k, j) for k in [kmin, kmax_stage] (k == kmin only when kmin > tile)
-    __shared__ uint64_t s[kBitonicTile];
-    const uint64_t base = static_cast<uint64_t>(blockIdx.x) * kBitonicTile;
-    s[threadIdx.x] = keys[base + threadIdx.x];
-    s[threadIdx.x + kBitonicThreads] = keys[base + threadIdx.x + kBitonicThreads];
-    __syncthreads();
-    for (uint64_t k = kmin; k <= kmax_stage; k <<= 1) {
-        uint64_t jstart = (k > static_cast<uint64_t>(kBitonicTile)) ? (kBitonicTile >> 1) : (k >> 1);
-        for (uint64_t j = jstart; j > 0; j >>= 1) {
-            // thread t handles pair (i, i+j) with i having bit j clear
-            uint64_t t = threadIdx.x;
-            uint64_t i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-            uint64_t gi = base + i;
-            bool asc = (gi & k) == 0;
-            uint64_t a = s[i], b = s[i + j];
-            if ((a > b) == asc) {
-                s[i] = b;
-                s[i + j] = a;
-            }
-            __syncthreads();
-        }
-    }
-    keys[base + threadIdx.x] = s[threadIdx.x];
-    keys[base + threadIdx.x + kBitonicThreads] = s[threadIdx.x + kBitonicThreads];
-}
-
-static __global__ void bitonic_global_kernel(uint64_t* __restrict__ keys, uint64_t N, uint64_t k, uint64_t j) {
-    for (uint64_t t = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; t < N / 2;
-         t += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        uint64_t i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-        bool asc = (i & k) == 0;
-        uint64_t a = keys[i], b = keys[i + j];
-        if ((a > b) == asc) {
-            keys[i] = b;
-            keys[i + j] = a;
-        }
-    }
-}
-
-inline cudaError_t bitonic_sort_u64(uint64_t* keys, uint64_t N, int num_sms, cudaStream_t st) {
-    // N is a power of two >= kBitonicTile
-    const unsigned nblk = static_cast<unsigned>(N / kBitonicTile);
-    bitonic_shared_kernel<<<nblk, kBitonicThreads, 0, st>>>(keys, 2, kBitonicTile);
-    for (uint64_t k = 2ull * kBitonicTile; k <= N; k <<= 1) {
-        for (uint64_t j = k >> 1; j >= static_cast<uint64_t>(kBitonicTile); j >>= 1)
-            bitonic_global_kernel<<<num_sms * 8, 512, 0, st>>>(keys, N, k, j);
-        bitonic_shared_kernel<<<nblk, kBitonicThreads, 0, st>>>(keys, k, k);
-    }
     return cudaGetLastError();
 }
 

@@ -147,12 +147,21 @@ typedef struct {
 /* Query options; a NULL pointer means all defaults (zeros). */
 typedef struct {
     int32_t chunk;       /* edges per work item of the middle join: 0 = default (16384), else a
-                            multiple of 32 in [32, 32768] (MHR_EINVAL otherwise) */
+                            multiple of 32 in [32, 32768] (MHR_EINVAL otherwise).  chunk and
+                            tile shape the join of graphs without a weight index */
     int32_t order;       /* order of intermediate vertices: 0 natural, 1 by score
                             bound, 2 by score bound refined inside bound levels by
-                            the learned slack prediction of `mlp` */
+                            the learned slack prediction of `mlp`.  On a graph with a
+                            weight index edges are read by their stored weights, which
+                            no order of the rows changes: only calls for the counters of
+                            order 0 use it there */
     int32_t prune;       /* 1 = skip work items, rows and middle edges whose provable
-                            score bound cannot reach the kept band (same result) */
+                            score bound cannot reach the kept band (same result).  0 =
+                            enumerate every middle edge when the call asks for the work
+                            counters (stats); without stats nothing that cannot change
+                            the result need be enumerated.  On a graph with a weight
+                            index calls with stats and prune 0 or order 0 run the join,
+                            all others the threshold search */
     int32_t precision;   /* middle-edge screen: 0 fp32 CUDA cores; 1 bf16 tensor-core
                             contraction with hi/lo split and fp32 accumulation (DistMult,
                             at most 16 relations); the fp64 rescoring keeps results exact */
@@ -174,7 +183,10 @@ typedef struct {
     int32_t reserved;
 } mhr_query_opts;
 
-/* Work counters of the last call (optional output). */
+/* Work counters of the last call (optional output).  With prune 1 on a graph with
+ * a weight index, edges_scanned counts every middle edge read (also those read
+ * only for a first threshold), hits the edges whose bound reached the kept band
+ * and paths the paths kept over them. */
 typedef struct {
     int64_t edges_scanned; /* middle-join CSR entries streamed */
     int64_t hits;          /* middle edges that joined both frontiers */
@@ -185,15 +197,18 @@ typedef struct {
     int64_t dense_queries; /* queries resolved by the exact (tie-heavy) path */
     double ms;             /* wall time of the call (synchronous calls only) */
     double ms_device;      /* device time of the whole launch sequence (CUDA events) */
-    double ms_join;        /* device time of the middle-join kernel (CUDA events) */
+    double ms_join;        /* device time of the middle-join or threshold-search kernel (CUDA events) */
     double ms_expand;      /* device time of the hop-1 / hop-3 expansion kernel (CUDA events;
-                              batched three-hop search only) */
+                              batched three-hop search only; 0 when the threshold search ran) */
 } mhr_stats;
 
 /*
  * Upload a graph and build its device indexes: the reverse CSR (in-edges of
- * each vertex, sorted by (source, relation)) and the norms behind the fp32
- * error bound.  Validates the description (MHR_EINVAL with a message on any
+ * each vertex, sorted by (source, relation)), the norms behind the fp32 error
+ * bound and, when it fits, the weight index: the fp32 weight of every edge and
+ * both adjacencies with each row sorted by it (36 bytes per edge, 80 per vertex;
+ * kept when it takes at most half of the device memory that is free beside the
+ * graph, and stays within the memory cap below).  Results do not depend on it.  Validates the description (MHR_EINVAL with a message on any
  * violation).  Synchronous; *out is NULL on failure, and a failed load has
  * released every device allocation it made.  A service that must keep the
  * graph within a memory budget sets the environment variable

@@ -385,7 +385,7 @@ def mhr_topk_paths(g: Graph, s: int, t: int, K: int, opts=None, with_stats: bool
     rc = lib.mhr_topk_paths(g.handle, ctypes.c_uint32(int(s) & 0xFFFFFFFF),
                             ctypes.c_uint32(int(t) & 0xFFFFFFFF), int(K), _ptr(out),
                             ctypes.byref(n_out), ctypes.byref(o) if o is not None else None,
-                            ctypes.byref(st))
+                            ctypes.byref(st) if with_stats else None)
     _check(rc)
     res = out[: n_out.value].copy()
     return (res, st.as_dict()) if with_stats else res

@@ -145,13 +145,98 @@ __device__ __forceinline__ int64_t row_of_edge(const int64_t* __restrict__ off, 
 // edge[i]: the CSR edges sorted by destination (stable, so a row is in
 // (source, relation) order)
 __global__ void k_fill_reverse(const uint32_t* __restrict__ edge, int64_t E, const uint32_t* __restrict__ src,
-                               const uint16_t* __restrict__ rel, uint32_t* __restrict__ rcol,
-                               uint16_t* __restrict__ rrel) {
+                               const uint16_t* __restrict__ rel, const float* __restrict__ w,
+                               uint32_t* __restrict__ rcol, uint16_t* __restrict__ rrel, float* __restrict__ rw) {
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < E; i += stride) {
         const uint32_t p = edge[i];
         rcol[i] = src[p];
         rrel[i] = rel[p];
+        if (rw) rw[i] = w[p];
+    }
+}
+
+// ---------------------------------------------------------------------------
+// weight index: rows sorted by fp32 edge weight, descending
+// ---------------------------------------------------------------------------
+__global__ void k_weight_keys(const float* __restrict__ w, int64_t E, uint32_t* __restrict__ key) {
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < E; i += stride)
+        key[i] = ~f2key(w[i]);
+}
+
+// key[i] = end[edge[i]]: the row (source or destination) of the i-th edge
+__global__ void k_row_keys(const uint32_t* __restrict__ edge, int64_t E, const uint32_t* __restrict__ end,
+                           uint32_t* __restrict__ key, uint32_t* __restrict__ copy) {
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < E; i += stride) {
+        const uint32_t e = edge[i];
+        key[i] = end[e];
+        copy[i] = e;
+    }
+}
+
+__global__ void k_fill_sorted(const uint32_t* __restrict__ edge, int64_t E, const uint32_t* __restrict__ far,
+                              const uint16_t* __restrict__ rel, const float* __restrict__ w, uint2* __restrict__ se,
+                              uint16_t* __restrict__ sr) {
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < E; i += stride) {
+        const uint32_t e = edge[i];
+        se[i] = make_uint2(far[e], __float_as_uint(w[e]));
+        sr[i] = rel[e];
+    }
+}
+
+__global__ void k_fill_records(const int64_t* __restrict__ off, int64_t n, const uint2* __restrict__ se,
+                               VertexRec* __restrict__ v, unsigned long long* __restrict__ sums) {
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) {
+        const int64_t lo = off[i], m = off[i + 1] - lo;
+        VertexRec r;
+        r.deg = static_cast<uint32_t>(m);
+        r.maxw = m > 0 ? __uint_as_float(se[lo].y) : 0.f;
+        r.row = static_cast<uint32_t>(lo);
+        r.maxp_key = 0u;
+        const int64_t at[4] = {4, 32, 256, 2048};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) r.rank[k] = __uint_as_float(m > at[k] ? se[lo + at[k]].y : 0xff800000u);
+        v[i] = r;
+        sums[i] = 0ull;
+    }
+}
+
+// p of every edge in row order, each row's largest p and the degrees summed over
+// it (one atomic per run of lanes in a row)
+__global__ void k_fill_potentials(const int64_t* __restrict__ off, int64_t n, int64_t E,
+                                  const uint32_t* __restrict__ col, const float* __restrict__ w, VertexRec* v,
+                                  float* __restrict__ p, unsigned long long* __restrict__ sums) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warp_id = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
+    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+    const int64_t steps = (E + 31) >> 5;
+    const int64_t s0 = steps * warp_id / nwarps, s1 = steps * (warp_id + 1) / nwarps;
+    if (s0 >= s1) return;  // warp-uniform
+    int64_t row = warp_row_search(off, n, s0 * 32, lane);
+    for (int64_t st = s0; st < s1; ++st) {
+        const int64_t i = st * 32 + lane;
+        const int64_t u = warp_rows_from(off, n, row, min(i, E - 1), lane);
+        row = __shfl_sync(0xffffffffu, u, 31);
+        uint32_t deg = 0u, key = 0u;
+        if (i < E) {
+            const uint2 f = *reinterpret_cast<const uint2*>(v + col[i]);  // deg and maxw
+            deg = f.x;
+            const float x = deg ? __fadd_rn(w[i], __uint_as_float(f.y)) : __int_as_float(0xff800000);
+            p[i] = x;
+            key = f2key(x);
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, i < E ? static_cast<uint32_t>(u) : 0xffffffffu);
+        const uint32_t km = __reduce_max_sync(peers, key);
+        const unsigned long long tot = (static_cast<unsigned long long>(__reduce_add_sync(peers, deg >> 16)) << 16) +
+                                       __reduce_add_sync(peers, deg & 0xffffu);
+        if (i < E && lane == __ffs(peers) - 1) {
+            atomicMax(&v[u].maxp_key, km);
+            if (tot) atomicAdd(&sums[u], tot);
+        }
     }
 }
 
@@ -437,6 +522,60 @@ mhr_status graph_alloc(mhr_graph* g, void** p, size_t bytes) {
     return MHR_OK;
 }
 
+// Device arrays of the weight index (36 bytes per edge and 80 per vertex)
+struct IndexArrays {
+    float *w, *rw, *p, *rp;
+    uint2 *se, *rse;
+    uint16_t *sr, *rsr;
+    VertexRec *vout, *vin;
+    unsigned long long *sout, *sin;
+};
+
+// The index is kept when it fits: within the graph's memory cap, and within
+// half of the device memory that is free once the graph itself is resident (the
+// rest stays for query plans).  A graph without one runs the joins that weigh
+// every hit.
+void alloc_index(mhr_graph* g, int64_t n, int64_t E, IndexArrays* ix) {
+    if (!E) return;
+    auto round = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t e2 = round(sizeof(uint16_t) * E), e4 = round(sizeof(uint32_t) * E), e8 = round(sizeof(uint2) * E),
+                 n8 = round(sizeof(unsigned long long) * n), nr = round(sizeof(VertexRec) * n);
+    const size_t total = 2 * (e2 + 2 * e4 + e8 + n8 + nr);
+    // still to come: the reverse adjacency, and (released later) the sort's scratch
+    const size_t later = static_cast<size_t>(E) * 6 + static_cast<size_t>(n) * 8;
+    if (g->memory_cap && g->alloc_bytes + total + later > g->memory_cap) return;
+    size_t avail = 0, all = 0;
+    if (cudaMemGetInfo(&avail, &all) != cudaSuccess || avail < later + static_cast<size_t>(E) * 4 ||
+        total > (avail - later - static_cast<size_t>(E) * 4) / 2) {
+        cudaGetLastError();
+        return;
+    }
+    char* p = nullptr;
+    if (cudaMalloc(reinterpret_cast<void**>(&p), total) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    g->allocations.push_back(p);
+    g->alloc_bytes += total;
+    auto take = [&](size_t bytes) {
+        char* q = p;
+        p += bytes;
+        return static_cast<void*>(q);
+    };
+    ix->w = static_cast<float*>(take(e4));
+    ix->rw = static_cast<float*>(take(e4));
+    ix->p = static_cast<float*>(take(e4));
+    ix->rp = static_cast<float*>(take(e4));
+    ix->se = static_cast<uint2*>(take(e8));
+    ix->rse = static_cast<uint2*>(take(e8));
+    ix->sr = static_cast<uint16_t*>(take(e2));
+    ix->rsr = static_cast<uint16_t*>(take(e2));
+    ix->vout = static_cast<VertexRec*>(take(nr));
+    ix->vin = static_cast<VertexRec*>(take(nr));
+    ix->sout = static_cast<unsigned long long*>(take(n8));
+    ix->sin = static_cast<unsigned long long*>(take(n8));
+}
+
 mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) {
     const int64_t n = desc->n_vertices, E = desc->n_edges;
     const int R = desc->n_relations, d = desc->dim;
@@ -513,6 +652,43 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
         return fail(MHR_EINVAL, "each row must be sorted by (col, rel) without repeated (col, rel)");
     if (herr[kErrNonFinite]) return fail(MHR_EINVAL, "an embedding value is NaN or infinite");
 
+    DevGraph& dg = g->dg;
+    dg.n = n;
+    dg.E = E;
+    dg.R = R;
+    dg.d = d;
+    dg.dtype = desc->emb_dtype;
+    dg.fn = desc->score_fn;
+    dg.gamma = desc->gamma;
+    dg.gamma32 = static_cast<float>(desc->gamma);
+    dg.off = off;
+    dg.col = col;
+    dg.rel = rel;
+    dg.vtypes = vt;
+    dg.vemb = vemb;
+    dg.remb = remb;
+    g->fn = desc->score_fn;
+
+    // --- fp32 edge weights: per-vertex maxima (pruning bounds), and the weights
+    // themselves when the index is kept
+    uint32_t *kout, *kin, *kout_r = nullptr, *kin_r = nullptr;
+    MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&kout), sizeof(uint32_t) * n));
+    MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&kin), sizeof(uint32_t) * n));
+    MHR_CUDA_TRY(cudaMemsetAsync(kout, 0, sizeof(uint32_t) * n, st));
+    MHR_CUDA_TRY(cudaMemsetAsync(kin, 0, sizeof(uint32_t) * n, st));
+    IndexArrays ix{};
+    alloc_index(g, n, E, &ix);
+    const int64_t nr = n * static_cast<int64_t>(R);
+    if (!ix.w && nr <= kMaxRelBoundEntries) {
+        // per (vertex, relation) bounds: the joins without an index weigh every hit
+        MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&kout_r), sizeof(uint32_t) * nr));
+        MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&kin_r), sizeof(uint32_t) * nr));
+        MHR_CUDA_TRY(cudaMemsetAsync(kout_r, 0, sizeof(uint32_t) * nr, st));
+        MHR_CUDA_TRY(cudaMemsetAsync(kin_r, 0, sizeof(uint32_t) * nr, st));
+    }
+    MHR_CUDA_TRY(launch_edge_w32(dg, nullptr, nullptr, nullptr, E, ix.w, kout, kin, kout_r, kin_r,
+                                 std::max(1, g->num_sms), st));
+
     // --- reverse CSR (in-edges of each vertex, rows sorted by (source, relation))
     int64_t* roff;
     uint32_t* rcol;
@@ -536,8 +712,29 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
             while (((n - 1) >> bits) != 0) ++bits;
             uint32_t* edge;
             MHR_CUDA_TRY(radix_sort_pairs(col, nullptr, static_cast<uint32_t>(E), bits, ss, &edge, st));
-            k_fill_reverse<<<grid, 256, 0, st>>>(edge, E, src, rel, rcol, rrel);
+            k_fill_reverse<<<grid, 256, 0, st>>>(edge, E, src, rel, ix.w, rcol, rrel, ix.rw);
             MHR_CUDA_TRY(cudaGetLastError());
+            if (ix.w) {
+                // All edges by weight, then (stable) by row: every row ends up in
+                // weight order, in both directions.
+                uint32_t* copy;
+                MHR_CUDA_TRY(tmp.alloc(&copy, sizeof(uint32_t) * E));
+                const uint32_t m = static_cast<uint32_t>(E);
+                k_weight_keys<<<grid, 256, 0, st>>>(ix.w, E, ss.key[0]);
+                MHR_CUDA_TRY(radix_sort_pairs(ss.key[0], nullptr, m, 32, ss, &edge, st));
+                uint32_t* key = edge == ss.val[0] ? ss.key[0] : ss.key[1];
+                k_row_keys<<<grid, 256, 0, st>>>(edge, E, src, key, copy);
+                MHR_CUDA_TRY(radix_sort_pairs(key, edge, m, bits, ss, &edge, st));
+                k_fill_sorted<<<grid, 256, 0, st>>>(edge, E, col, rel, ix.w, ix.se, ix.sr);
+                k_row_keys<<<grid, 256, 0, st>>>(copy, E, col, ss.key[0], ss.val[0]);
+                MHR_CUDA_TRY(radix_sort_pairs(ss.key[0], ss.val[0], m, bits, ss, &edge, st));
+                k_fill_sorted<<<grid, 256, 0, st>>>(edge, E, src, rel, ix.w, ix.rse, ix.rsr);
+                k_fill_records<<<grid, 256, 0, st>>>(off, n, ix.se, ix.vout, ix.sout);
+                k_fill_records<<<grid, 256, 0, st>>>(roff, n, ix.rse, ix.vin, ix.sin);
+                k_fill_potentials<<<grid, 256, 0, st>>>(off, n, E, col, ix.w, ix.vout, ix.p, ix.sout);
+                k_fill_potentials<<<grid, 256, 0, st>>>(roff, n, E, rcol, ix.rw, ix.vin, ix.rp, ix.sin);
+                MHR_CUDA_TRY(cudaGetLastError());
+            }
         }
         // the scan wrote n_dev-long output plus the total at roff[n]
         MHR_CUDA_TRY(cudaStreamSynchronize(st));
@@ -572,25 +769,21 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
         g->max_in_deg = std::max(g->max_in_deg, g->h_roff[u + 1] - g->h_roff[u]);
     }
 
-    DevGraph& dg = g->dg;
-    dg.n = n;
-    dg.E = E;
-    dg.R = R;
-    dg.d = d;
-    dg.dtype = desc->emb_dtype;
-    dg.fn = desc->score_fn;
-    dg.gamma = desc->gamma;
-    dg.gamma32 = static_cast<float>(desc->gamma);
-    dg.off = off;
-    dg.col = col;
-    dg.rel = rel;
     dg.roff = roff;
     dg.rcol = rcol;
     dg.rrel = rrel;
-    dg.vtypes = vt;
-    dg.vemb = vemb;
-    dg.remb = remb;
-    g->fn = desc->score_fn;
+    dg.w = ix.w;
+    dg.rw = ix.rw;
+    dg.se = ix.se;
+    dg.sr = ix.sr;
+    dg.rse = ix.rse;
+    dg.rsr = ix.rsr;
+    dg.p = ix.p;
+    dg.rp = ix.rp;
+    dg.vout = ix.vout;
+    dg.vin = ix.vin;
+    dg.sout = ix.sout;
+    dg.sin = ix.sin;
     compute_bounds(g);
     if (g->fn == MHR_SCORE_DISTMULT) {
         const int64_t cnt = static_cast<int64_t>(R) * d;
@@ -599,24 +792,9 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
             remb, desc->emb_dtype, cnt, g->wsplit, g->wsplit + cnt);
         MHR_CUDA_TRY(cudaGetLastError());
     }
-    // per-vertex bounds on the fp32 weight of adjacent edges (bound pruning),
-    // and per (vertex, relation) bounds when n x R entries stay within
-    // kMaxRelBoundEntries (4 bytes each, two tables)
+    // per-vertex (and, without the index, per (vertex, relation)) bounds on the
+    // fp32 weight of adjacent edges, for bound pruning
     {
-        uint32_t *kout, *kin, *kout_r = nullptr, *kin_r = nullptr;
-        MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&kout), sizeof(uint32_t) * n));
-        MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&kin), sizeof(uint32_t) * n));
-        MHR_CUDA_TRY(cudaMemsetAsync(kout, 0, sizeof(uint32_t) * n, st));
-        MHR_CUDA_TRY(cudaMemsetAsync(kin, 0, sizeof(uint32_t) * n, st));
-        const int64_t nr = n * static_cast<int64_t>(R);
-        if (nr <= kMaxRelBoundEntries) {
-            MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&kout_r), sizeof(uint32_t) * nr));
-            MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&kin_r), sizeof(uint32_t) * nr));
-            MHR_CUDA_TRY(cudaMemsetAsync(kout_r, 0, sizeof(uint32_t) * nr, st));
-            MHR_CUDA_TRY(cudaMemsetAsync(kin_r, 0, sizeof(uint32_t) * nr, st));
-        }
-        MHR_CUDA_TRY(launch_edge_w32(dg, nullptr, nullptr, nullptr, E, nullptr, kout, kin, kout_r, kin_r,
-                                     std::max(1, g->num_sms), st));
         k_maxw_finish<<<grid, 256, 0, st>>>(kout, n, 2.0 * g->eps32_edge);
         k_maxw_finish<<<grid, 256, 0, st>>>(kin, n, 2.0 * g->eps32_edge);
         if (kout_r) {

@@ -34,6 +34,15 @@ mhr_status cuda_fail(cudaError_t e, const char* what);
 // ---------------------------------------------------------------------------
 // device view of a loaded graph (POD, passed by value to kernels)
 // ---------------------------------------------------------------------------
+// one vertex's row in the weight index (one 32-byte sector)
+struct __align__(32) VertexRec {
+    uint32_t deg;
+    float maxw;         // its largest weight (0 when it has no edge)
+    uint32_t row;       // first position in the sorted adjacency
+    uint32_t maxp_key;  // order key of the largest p of its edges, 0 when it has none
+    float rank[4];      // weights at ranks 4, 32, 256 and 2048 (from 0), -inf past its end
+};
+
 struct DevGraph {
     int64_t n, E;
     int32_t R, d, dtype, fn;
@@ -57,6 +66,20 @@ struct DevGraph {
     // n x R exceeds kMaxRelBoundEntries
     const float* maxw_out_r;
     const float* maxw_in_r;
+    // weight index (all NULL when the graph has none): the fp32 weight of every
+    // edge, and the adjacency in both directions with each row sorted by it
+    const float* w;        // [E] CSR order
+    const float* rw;       // [E] reverse CSR order
+    const float* p;        // [E] w + the largest weight out of the destination (-inf: it has no out-edge)
+    const float* rp;       // [E] rw + the largest weight into the source
+    const uint2* se;       // [E] out-rows, weight descending: (destination, weight bits)
+    const uint16_t* sr;    // [E] their relation ids
+    const uint2* rse;      // [E] in-rows, weight descending: (source, weight bits)
+    const uint16_t* rsr;   // [E]
+    const VertexRec* vout; // [n] out-rows
+    const VertexRec* vin;  // [n] in-rows
+    const unsigned long long* sout;  // [n] out-degrees summed over the out-row
+    const unsigned long long* sin;   // [n] in-degrees summed over the in-row
 };
 
 constexpr int64_t kMaxRelBoundEntries = int64_t(1) << 29;  // 2 GiB per table

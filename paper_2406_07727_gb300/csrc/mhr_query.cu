@@ -5,7 +5,16 @@
 // order score descending, (u, r1, v, r2, r3) ascending.  The paper's CPU
 // design (Sec. 3.3, Alg. 2-4; Sec. 5, Alg. 6-7) keeps thread-private k-heaps
 // and merges them with a barrier tree; here the same exact result comes from
-// a meet-in-the-middle join sized for one GB300:
+// one of two meet-in-the-middle searches:
+//
+// On a graph with a weight index, the threshold search (mhr_search.cuh): one
+// launch, one block per query, which reads only the middle edges whose stored
+// weight can still matter.  Its candidates go through the rescoring and merge
+// below.  Queries it hands back (ties, prefixes too long for one block) run
+// through the join as a conditional part of the same CUDA graph.
+//
+// Otherwise (no index, label runs, or a call that asks for the counters of a full
+// enumeration), the join, sized for one GB300:
 //
 //   expand   hop-1 row of s and hop-3 (reverse) row of t, fp32 weights,
 //            distinct frontier vertices with their best weight; S_f = sum of
@@ -37,6 +46,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstddef>
 #include <cstring>
@@ -48,29 +58,17 @@
 #include "mhr_query.cuh"
 #include "mhr_mlp_tc.cuh"
 #include "mhr_score.cuh"
+#include "mhr_search.cuh"
 #include "mhr_util.cuh"
 
 namespace mhr {
 
 constexpr unsigned FULL = 0xffffffffu;
 
-__device__ __forceinline__ unsigned lanemask_lt() {
-    unsigned m;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-    return m;
-}
 __device__ __forceinline__ unsigned lanemask_le() {
     unsigned m;
     asm("mov.u32 %0, %%lanemask_le;" : "=r"(m));
     return m;
-}
-
-__device__ __forceinline__ float neg_inf() { return __int_as_float(0xff800000); }
-
-// thr - 2E rounded toward -inf, as float (conservative keep threshold)
-__device__ __forceinline__ float keep_threshold(uint32_t key, double two_err) {
-    if (key == 0u) return neg_inf();
-    return __double2float_rd(__dsub_rd(static_cast<double>(key2f(key)), two_err));
 }
 
 // path order: 1 if a ranks strictly before b
@@ -110,62 +108,16 @@ __device__ void block_sort_paths(mhr_path* a, int m) {
     }
 }
 
-// K-th largest order key among n keys (1 <= K <= n) by 4-pass radix select.
-// key_at(i) gives key i; all threads call; hist has 256 slots.
-template <typename KeyAt>
-__device__ uint32_t block_select_kth(KeyAt key_at, int64_t n, int K, uint32_t* hist, uint32_t* bcast) {
-    uint32_t prefix = 0, mask = 0;
-    uint32_t remaining = static_cast<uint32_t>(K);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int pass = 0; pass < 4; ++pass) {
-        const int shift = 24 - 8 * pass;
-        for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
-        __syncthreads();
-        for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-            uint32_t k = key_at(i);
-            if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1u);
-        }
-        __syncthreads();
-        if (wid == 0) {
-            // lane l owns bins 255-8l .. 248-8l (descending)
-            uint32_t c = 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) c += hist[255 - 8 * lane - j];
-            uint32_t cum = warp_incl_scan(c);
-            unsigned b = __ballot_sync(FULL, cum >= remaining);
-            int L = __ffs(b) - 1;
-            if (lane == L) {
-                uint32_t before = cum - c;
-                for (int j = 0; j < 8; ++j) {
-                    uint32_t bin = 255 - 8 * lane - j;
-                    uint32_t h = hist[bin];
-                    if (before + h >= remaining) {
-                        bcast[0] = prefix | (bin << shift);
-                        bcast[1] = remaining - before;
-                        break;
-                    }
-                    before += h;
-                }
-            }
-        }
-        __syncthreads();
-        prefix = bcast[0];
-        remaining = bcast[1];
-        mask |= 255u << shift;
-        __syncthreads();
-    }
-    return prefix;
-}
-
 // ===========================================================================
 // frontier expansion
 // ===========================================================================
-__global__ void k_init(const PlanDev* __restrict__ P, DevGraph g) {
+// redo: only the queries the threshold search handed back are answered
+__global__ void k_init(const PlanDev* __restrict__ P, DevGraph g, bool redo) {
     const int nq = P->nq;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     for (int q = tid; q < nq; q += gridDim.x * blockDim.x) {
         const uint32_t s = P->S[q], t = P->T[q];
-        P->status[q] = (s < g.n && t < g.n && s != t) ? 0 : 1;
+        P->status[q] = redo ? (P->status[q] == 3 ? 0 : 2) : ((s < g.n && t < g.n && s != t) ? 0 : 1);
         P->thr_g[q] = 0u;
         P->qmax[2 * q] = 0u;
         P->qmax[2 * q + 1] = 0u;
@@ -175,9 +127,8 @@ __global__ void k_init(const PlanDev* __restrict__ P, DevGraph g) {
         P->pool_cnt[q] = 0;
         P->band_cnt[q] = 0;
         P->chain_cnt[q] = 0;
-        P->n_out[q] = 0;
+        if (!redo) P->n_out[q] = 0;
     }
-    if (tid < kCntCount) P->counters[tid] = 0ull;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int c = tid; c < P->grid; c += gridDim.x * blockDim.x) P->cursors[c] = 0ull;
     for (int c = tid; c < (P->grid + 31) / 32; c += gridDim.x * blockDim.x) P->drained[c] = 0u;
@@ -241,6 +192,7 @@ __device__ __forceinline__ void slot_commit(const PlanDev* __restrict__ P, const
         // A vertex with no scan edges can neither be scanned nor be hit, so it
         // never lies on a path: it is dropped from the distinct list.
         bool head = !excl && o.sdeg > 0 && (o.k == 0 || o.prev != vtx);
+        if (P->status[o.q] != 0) head = false;  // answered already
         // vertex partition: this call owns the paths whose hop-1 vertex u it owns
         if (sideA && P->part_count > 1 && vtx % static_cast<uint32_t>(P->part_count) !=
                                               static_cast<uint32_t>(P->part_index))
@@ -2022,6 +1974,100 @@ __global__ void __launch_bounds__(kMidThreads, 1) k_middle(const PlanDev* __rest
 }
 
 // ===========================================================================
+// threshold search over the weight index (mhr_search.cuh)
+// ===========================================================================
+constexpr int kSrSpill = 15360;  // candidates past kSrCand, per block
+
+// Persistent blocks take queries, largest rows first; a query's candidates (all
+// paths that can be among its K best) become its band, and the fp64 sums the band
+// needs are listed: every middle edge, each hop-1 and hop-3 edge once.
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_search(const PlanDev* __restrict__ P, DevGraph g) {
+    SearchSmem<NT>& sm = sr_smem<NT>();
+    __shared__ int s_q;
+    const int nq = P->nq, K = P->K, band_cap = P->band_cap;
+    for (;;) {
+        if (threadIdx.x == 0) {
+            const unsigned long long i = atomicAdd(&P->counters[kCntItem], 1ull);
+            s_q = i < static_cast<unsigned long long>(nq) ? static_cast<int>(P->qord[i]) : -1;
+        }
+        __syncthreads();
+        const int q = s_q;
+        if (q < 0) break;
+        const uint32_t s = P->S[q], t = P->T[q];
+        const bool valid = s < g.n && t < g.n && s != t;
+        if (threadIdx.x == 0) {
+            sm.s = s;
+            sm.t = t;
+            sm.K = K;
+            sm.part_count = P->part_count;
+            sm.part_index = P->part_index;
+            sm.cons = P->cons;
+            sm.R = g.R;
+            sm.two_err = 2.0 * P->err_path;
+            sm.spill = P->spill + static_cast<int64_t>(blockIdx.x) * kSrSpill;
+            sm.spill_queue = P->spill_queue + static_cast<int64_t>(blockIdx.x) * kSrSpillQueue;
+            sm.cap = kSrCand + kSrSpill;
+            sm.redo = 0;
+            sm.cand_cnt = 0;
+        }
+        __syncthreads();
+        if (valid) search_query<NT>(g, static_cast<unsigned long long>(P->heavy));
+        __syncthreads();
+        const int m = sm.cand_cnt;
+        const bool redo = valid && (sm.redo || m > band_cap);
+        const int nb = valid && !redo ? m : 0;
+        Cand* band = P->band_cand + static_cast<int64_t>(q) * band_cap;
+        const int64_t a0 = P->a_off[q], c0 = P->totA + P->c_off[q];
+        for (int i = threadIdx.x; i < nb; i += NT) {
+            const Cand c = sr_cand(sm, i);
+            band[i] = c;
+            P->w64own[a0 + c.a_idx] = 0;
+            P->w64own[c0 + c.c_idx] = 0;
+        }
+        __syncthreads();
+        uint32_t* ch = P->chains + static_cast<int64_t>(q) * 3 * band_cap;
+        int nch = 0;
+        for (int base = 0; base < nb; base += NT) {
+            const int i = base + threadIdx.x;
+            int n = 0;
+            bool o1 = false, o3 = false;
+            Cand c;
+            if (i < nb) {
+                c = sr_cand(sm, i);
+                o1 = atomicExch(&P->w64own[a0 + c.a_idx], 1) == 0;
+                o3 = atomicExch(&P->w64own[c0 + c.c_idx], 1) == 0;
+                n = 1 + (o1 ? 1 : 0) + (o3 ? 1 : 0);
+            }
+            int tot;
+            int pos = nch + block_excl_scan(n, reinterpret_cast<int*>(sm.red), &tot);
+            if (i < nb) {
+                ch[pos++] = (2u << 30) | static_cast<uint32_t>(i);
+                if (o1) ch[pos++] = (0u << 30) | c.a_idx;
+                if (o3) ch[pos++] = (1u << 30) | c.c_idx;
+            }
+            nch += tot;
+        }
+        if (threadIdx.x == 0) {
+            P->status[q] = !valid ? 1 : (redo ? 3 : 0);
+            P->dense[q] = 0;
+            P->band_cnt[q] = nb;
+            P->chain_cnt[q] = nch;
+            if (redo) atomicAdd(&P->counters[kCntRedo], 1ull);
+            if (valid && !redo) {
+                atomicAdd(&P->counters[kCntRescored], static_cast<unsigned long long>(nb));
+                atomicAdd(&P->counters[kCntCands], static_cast<unsigned long long>(m));
+                atomicAdd(&P->counters[kCntScanned], sm.scanned);
+                atomicAdd(&P->counters[kCntHits], sm.hits);
+                atomicAdd(&P->counters[kCntPaths], sm.paths);
+                if (sm.near_edges > sm.scanned) atomicAdd(&P->counters[kCntPruned], sm.near_edges - sm.scanned);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// ===========================================================================
 // merge: exact K-th fp32 score, band, fp64 rescoring, final order
 // ===========================================================================
 __global__ void __launch_bounds__(1024) k_merge1(const PlanDev* __restrict__ P) {
@@ -2213,13 +2259,17 @@ __global__ void __launch_bounds__(kRsWarps * 32) k_rescore(const PlanDev* __rest
     }
 }
 
-__global__ void __launch_bounds__(1024) k_merge2(const PlanDev* __restrict__ P, DevGraph g) {
+// with `redo`, its condition (a conditional graph node: the join of the queries
+// the threshold search handed back) is set when there are any
+__global__ void __launch_bounds__(1024) k_merge2(const PlanDev* __restrict__ P, DevGraph g,
+                                                 cudaGraphConditionalHandle redo, bool has_redo) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     mhr_path* buf = reinterpret_cast<mhr_path*>(smem_raw);
     const int K = P->K;
+    if (has_redo && blockIdx.x == 0 && threadIdx.x == 0 && P->counters[kCntRedo]) cudaGraphSetConditional(redo, 1u);
     for (int q = blockIdx.x; q < P->nq; q += gridDim.x) {
         if (P->status[q] != 0) {
-            if (threadIdx.x == 0) P->n_out[q] = -1;
+            if (threadIdx.x == 0 && P->status[q] == 1) P->n_out[q] = -1;
             continue;
         }
         if (P->dense[q]) continue;
@@ -2448,7 +2498,7 @@ struct Plan {
     int expand_per_sm = 8;  // resident expansion blocks per SM
     void (*expand_fn)(const PlanDev*, DevGraph) = nullptr;  // the expansion kernel for the graph's rows
     PlanDev h{};
-    unsigned char* dregion = nullptr;  // [PlanDev][S][T][a_off][c_off]
+    unsigned char* dregion = nullptr;  // [PlanDev][S][T][a_off][c_off][constraints][counters][query order]
     size_t region_bytes = 0;
     unsigned char* pin = nullptr;      // pinned host mirror of dregion
     std::vector<void*> fixed;
@@ -2456,7 +2506,10 @@ struct Plan {
     int64_t slot_cap = 0;
     void* item_mem = nullptr;
     void* far_mem = nullptr;
-    cudaGraphExec_t exec[3] = {nullptr, nullptr, nullptr};
+    cudaGraphExec_t exec[3] = {nullptr, nullptr, nullptr};  // expansion and order, join, merge
+    cudaGraphExec_t exec_search = nullptr;                   // threshold search, with the above as its conditional part
+    int search_threads = 512, search_grid = 1;
+    bool searched = false;  // the last call ran exec_search
     cudaStream_t cap = nullptr;
     cudaEvent_t h2d_done = nullptr;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // before / join / after / end
@@ -2468,6 +2521,8 @@ struct Plan {
                 cudaGraphExecDestroy(x);
                 x = nullptr;
             }
+        if (exec_search) cudaGraphExecDestroy(exec_search);
+        exec_search = nullptr;
     }
     ~Plan() {
         drop_graphs();
@@ -2501,7 +2556,7 @@ void destroy_plans(mhr_graph* g) {
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct RegionLayout {
-    size_t off_S, off_T, off_a, off_c, off_cons, total;
+    size_t off_S, off_T, off_a, off_c, off_cons, off_cnt, off_ord, total;
 };
 
 // bytes of the constraint flags: three relation sets and two type sets
@@ -2520,6 +2575,10 @@ static RegionLayout region_layout(int nq, int R) {
     o = align_up(o + sizeof(int64_t) * (nq + 1), 256);
     L.off_cons = o;
     o = align_up(o + cons_bytes(R), 256);
+    L.off_cnt = o;
+    o = align_up(o + sizeof(unsigned long long) * kCntCount, 256);
+    L.off_ord = o;
+    o = align_up(o + sizeof(uint32_t) * nq, 256);
     L.total = o;
     return L;
 }
@@ -2536,6 +2595,7 @@ static mhr_status plan_alloc(Plan* p, T** out, size_t count) {
 
 static size_t mid_smem_bytes() { return sizeof(MidSmem); }
 static_assert(sizeof(MidSmem) <= 232448, "the join's shared memory fits one CTA per SM (227 KB)");
+static_assert(2 * sizeof(SearchSmem<512>) <= 230000, "two 512-thread search blocks per SM");
 static size_t exact_smem_bytes() { return sizeof(ExactSmem); }
 static size_t merge2_smem_bytes(int band_cap) {
     int m = 2;
@@ -2641,17 +2701,19 @@ static mhr_status ensure_items(Plan* p, int64_t cap) {
     return MHR_OK;
 }
 
-static cudaError_t launch_part(Plan* p, const mhr_graph* G, cudaStream_t st, int part) {
+// redo: the join as the conditional part of the threshold search (no event
+// records, which a conditional body cannot hold; queries answered already are skipped)
+static cudaError_t launch_part(Plan* p, const mhr_graph* G, cudaStream_t st, int part, bool redo) {
     const PlanDev* d = reinterpret_cast<const PlanDev*>(p->dregion);
     const int sms = std::max(1, G->num_sms);
     const DevGraph& g = G->dg;
     const int64_t* nX = reinterpret_cast<const int64_t*>(p->dregion + offsetof(PlanDev, X));
     if (part == 0) {
-        k_init<<<sms * 2, 256, 0, st>>>(d, g);
-        cudaError_t ee = cudaEventRecordWithFlags(p->ev_x[0], st, cudaEventRecordExternal);
+        k_init<<<sms * 2, 256, 0, st>>>(d, g, redo);
+        cudaError_t ee = redo ? cudaSuccess : cudaEventRecordWithFlags(p->ev_x[0], st, cudaEventRecordExternal);
         if (ee != cudaSuccess) return ee;
         p->expand_fn<<<sms * p->expand_per_sm, 256, 0, st>>>(d, g);
-        ee = cudaEventRecordWithFlags(p->ev_x[1], st, cudaEventRecordExternal);
+        ee = redo ? cudaSuccess : cudaEventRecordWithFlags(p->ev_x[1], st, cudaEventRecordExternal);
         if (ee != cudaSuccess) return ee;
         cudaError_t e = device_excl_scan<uint32_t>(p->h.flag, nX, p->h.partials, p->h.scan1, st);
         if (e != cudaSuccess) return e;
@@ -2690,7 +2752,7 @@ static cudaError_t launch_part(Plan* p, const mhr_graph* G, cudaStream_t st, int
     } else {
         k_merge1<<<std::min(p->nq, sms * 2), 1024, 0, st>>>(d);
         k_rescore<<<sms * 4, kRsWarps * 32, 0, st>>>(d, g);
-        k_merge2<<<std::min(p->nq, sms * 2), 1024, merge2_smem_bytes(p->h.band_cap), st>>>(d, g);
+        k_merge2<<<std::min(p->nq, sms * 2), 1024, merge2_smem_bytes(p->h.band_cap), st>>>(d, g, 0, false);
         k_exact<<<std::min(p->nq, sms * 2), 1024, exact_smem_bytes(), st>>>(d, g);
     }
     return cudaGetLastError();
@@ -2701,7 +2763,7 @@ static mhr_status capture(Plan* p, const mhr_graph* G) {
     for (int part = 0; part < 3; ++part) {
         cudaGraph_t graph = nullptr;
         MHR_CUDA_TRY(cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = launch_part(p, G, p->cap, part);
+        cudaError_t e = launch_part(p, G, p->cap, part, false);
         cudaError_t e2 = cudaStreamEndCapture(p->cap, &graph);
         if (e != cudaSuccess || e2 != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
@@ -2718,8 +2780,74 @@ static mhr_status capture(Plan* p, const mhr_graph* G) {
     return MHR_OK;
 }
 
+// search, rescoring and merge, then the whole join as a conditional node that
+// runs when queries were handed back
+static cudaError_t build_search_graph(Plan* p, const mhr_graph* G, cudaGraph_t graph) {
+    const PlanDev* d = reinterpret_cast<const PlanDev*>(p->dregion);
+    const int sms = std::max(1, G->num_sms);
+    const DevGraph& g = G->dg;
+    cudaStream_t st = p->cap;
+    cudaGraphConditionalHandle handle;
+    cudaError_t e = cudaGraphConditionalHandleCreate(&handle, graph, 0, cudaGraphCondAssignDefault);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamBeginCaptureToGraph(st, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    cudaError_t ee = cudaEventRecordWithFlags(p->ev_x[0], st, cudaEventRecordExternal);
+    if (p->search_threads == 512) k_search<512><<<p->search_grid, 512, sizeof(SearchSmem<512>), st>>>(d, g);
+    else k_search<1024><<<p->search_grid, 1024, sizeof(SearchSmem<1024>), st>>>(d, g);
+    if (ee == cudaSuccess) ee = cudaEventRecordWithFlags(p->ev_x[1], st, cudaEventRecordExternal);
+    k_rescore<<<sms * 4, kRsWarps * 32, 0, st>>>(d, g);
+    k_merge2<<<std::min(p->nq, sms * 2), 1024, merge2_smem_bytes(p->h.band_cap), st>>>(d, g, handle, true);
+    if (ee == cudaSuccess) ee = cudaGetLastError();
+    // the capture's last node carries the dependency of the conditional one
+    cudaStreamCaptureStatus status;
+    const cudaGraphNode_t* deps = nullptr;
+    const cudaGraphEdgeData* edges = nullptr;
+    size_t n_deps = 0;
+    if (ee == cudaSuccess)
+        ee = cudaStreamGetCaptureInfo(st, &status, nullptr, nullptr, &deps, &edges, &n_deps);
+    std::vector<cudaGraphNode_t> last(deps, deps + n_deps);
+    e = cudaStreamEndCapture(st, &graph);
+    if (ee != cudaSuccess) return ee;
+    if (e != cudaSuccess) return e;
+    cudaGraphNodeParams cp{};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = handle;
+    cp.conditional.type = cudaGraphCondTypeIf;
+    cp.conditional.size = 1;
+    cudaGraphNode_t node;
+    e = cudaGraphAddNode(&node, graph, last.data(), nullptr, last.size(), &cp);
+    if (e != cudaSuccess) return e;
+    cudaGraph_t body = cp.conditional.phGraph_out[0];
+    e = cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    ee = cudaSuccess;
+    for (int part = 0; part < 3 && ee == cudaSuccess; ++part) ee = launch_part(p, G, st, part, true);
+    e = cudaStreamEndCapture(st, &body);
+    return ee != cudaSuccess ? ee : e;
+}
+
+static mhr_status capture_search(Plan* p, const mhr_graph* G) {
+    if (p->exec_search) return MHR_OK;
+    cudaGraph_t graph = nullptr;
+    MHR_CUDA_TRY(cudaGraphCreate(&graph, 0));
+    cudaError_t e = build_search_graph(p, G, graph);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&p->exec_search, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {
+        p->exec_search = nullptr;
+        return cuda_fail(e, "search graph");
+    }
+    return MHR_OK;
+}
+
 static cudaError_t launch_graphs(Plan* p, cudaStream_t st) {
     cudaError_t e;
+    if (p->searched) {
+        if ((e = cudaEventRecord(p->ev[0], st)) != cudaSuccess) return e;
+        if ((e = cudaGraphLaunch(p->exec_search, st)) != cudaSuccess) return e;
+        return cudaEventRecord(p->ev[3], st);
+    }
     for (int part = 0; part < 3; ++part) {
         if ((e = cudaEventRecord(p->ev[part], st)) != cudaSuccess) return e;
         if ((e = cudaGraphLaunch(p->exec[part], st)) != cudaSuccess) return e;
@@ -2793,7 +2921,15 @@ static mhr_status make_plan(mhr_graph* G, int nq, int K, int chunk, int precisio
     if ((rc = plan_alloc(p, &h.chain_cnt, nq)) != MHR_OK) return bail(rc);
     if ((rc = plan_alloc(p, &h.out, static_cast<size_t>(nq) * K)) != MHR_OK) return bail(rc);
     if ((rc = plan_alloc(p, &h.n_out, nq)) != MHR_OK) return bail(rc);
-    if ((rc = plan_alloc(p, &h.counters, kCntCount)) != MHR_OK) return bail(rc);
+    if (G->dg.w) {
+        // enough queries for two blocks on every SM: 512 threads each; else one
+        // 1,024-thread block per query shortens its phases
+        p->search_threads = nq > p->grid ? 512 : 1024;
+        p->search_grid = std::min(nq, p->search_threads == 512 ? 2 * p->grid : p->grid);
+        if ((rc = plan_alloc(p, &h.spill, static_cast<size_t>(p->search_grid) * kSrSpill)) != MHR_OK) return bail(rc);
+        if ((rc = plan_alloc(p, &h.spill_queue, static_cast<size_t>(p->search_grid) * kSrSpillQueue)) != MHR_OK)
+            return bail(rc);
+    }
     if ((rc = plan_alloc(p, &h.partials, kScanPartials)) != MHR_OK) return bail(rc);
     if (cudaMemset(h.partials, 0, sizeof(int64_t) * kScanPartials) != cudaSuccess)
         return bail(cuda_fail(cudaGetLastError(), "cudaMemset (scan counter)"));
@@ -2808,6 +2944,8 @@ static mhr_status make_plan(mhr_graph* G, int nq, int K, int chunk, int precisio
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMallocHost (plan region)"));
     h.S = reinterpret_cast<const uint32_t*>(p->dregion + L.off_S);
     h.T = reinterpret_cast<const uint32_t*>(p->dregion + L.off_T);
+    h.counters = reinterpret_cast<unsigned long long*>(p->dregion + L.off_cnt);
+    h.qord = reinterpret_cast<const uint32_t*>(p->dregion + L.off_ord);
     h.a_off = reinterpret_cast<const int64_t*>(p->dregion + L.off_a);
     h.c_off = reinterpret_cast<const int64_t*>(p->dregion + L.off_c);
     e = cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking);
@@ -2834,7 +2972,13 @@ static mhr_status make_plan(mhr_graph* G, int nq, int K, int chunk, int precisio
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k_middle<8, true, true>, a, sb);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k_middle<8, false, true>, a, sb);
     }
-    if (e != cudaSuccess) return bail(cuda_fail(e, "cudaFuncSetAttribute (middle join)"));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_search<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(sizeof(SearchSmem<512>)));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_search<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(sizeof(SearchSmem<1024>)));
+    if (e != cudaSuccess) return bail(cuda_fail(e, "cudaFuncSetAttribute (middle join, search)"));
     {
         // one resident wave of the grid-stride expansion kernel
         int nb = 0;
@@ -2877,7 +3021,8 @@ static mhr_status get_plan(mhr_graph* G, int nq, int K, int chunk, int precision
 }
 
 static mhr_status run_batch(mhr_graph* G, int nq, const uint32_t* hS, const uint32_t* hT, int K,
-                            const mhr_query_opts* opts, cudaStream_t st, Plan** plan_out, bool label = false) {
+                            const mhr_query_opts* opts, cudaStream_t st, Plan** plan_out, bool counters,
+                            bool label = false) {
     int chunk = (opts && opts->chunk > 0) ? opts->chunk : kDefaultChunk;
     if (chunk > kMaxChunk || chunk < 32 || (chunk & 31))
         return fail(MHR_EINVAL, "opts->chunk must be a multiple of 32 in [32, 32768]");
@@ -2941,6 +3086,10 @@ static mhr_status run_batch(mhr_graph* G, int nq, const uint32_t* hS, const uint
         p->h.mlp.w2 = m->w2;
         p->h.mlp.b2 = m->b2;
     }
+    // The threshold search answers every call on a graph with a weight index,
+    // except label runs and those that ask for the counters of a full enumeration
+    // or of the natural order (stats with prune 0 or order 0).
+    const bool searched = G->dg.w && !label && (!counters || (p->h.prune && p->h.order));
     p->h.label = label ? 1 : 0;
     if (label && (p->h.prune || p->h.order)) return fail(MHR_EINVAL, "label runs use the plain search");
     // vertex partition of the paths by their hop-1 vertex
@@ -2965,11 +3114,30 @@ static mhr_status run_batch(mhr_graph* G, int nq, const uint32_t* hS, const uint
             for (int y = 0; y < 256; ++y) f[3 * R + h * 256 + y] = ty[h] ? (ty[h][y] != 0) : 1;
         p->h.cons = p->dregion + L.off_cons;
     }
+    std::memset(p->pin + L.off_cnt, 0, sizeof(unsigned long long) * kCntCount);
+    p->searched = searched;
+    if (searched) {
+        // queries handed back go through the pruned join, rows by their bound
+        p->h.prune = 1;
+        if (p->h.order == 0) p->h.order = 1;
+        p->h.heavy = int64_t(1) << 22;
+        // largest rows first (by powers of two), so that no long query starts last
+        uint32_t* ord = reinterpret_cast<uint32_t*>(p->pin + L.off_ord);
+        uint32_t first[65] = {0};
+        auto level = [&](int q) {
+            const uint64_t x = static_cast<uint64_t>(pa[q + 1] - pa[q]) + static_cast<uint64_t>(pc[q + 1] - pc[q]);
+            return x ? __builtin_clzll(x) : 64;
+        };
+        for (int q = 0; q < nq; ++q)
+            if (level(q) < 64) ++first[level(q) + 1];
+        for (int i = 1; i <= 64; ++i) first[i] += first[i - 1];
+        for (int q = 0; q < nq; ++q) ord[first[level(q)]++] = static_cast<uint32_t>(q);
+    }
     std::memcpy(p->pin, &p->h, sizeof(PlanDev));
     MHR_CUDA_TRY(cudaMemcpyAsync(p->dregion, p->pin, L.total, cudaMemcpyHostToDevice, st));
     MHR_CUDA_TRY(cudaEventRecord(p->h2d_done, st));
     p->h2d_pending = true;
-    MHR_TRY(capture(p, G));
+    MHR_TRY(searched ? capture_search(p, G) : capture(p, G));
     MHR_CUDA_TRY(launch_graphs(p, st));
     *plan_out = p;
     return MHR_OK;
@@ -2988,10 +3156,15 @@ static mhr_status read_stats(Plan* p, cudaStream_t st, mhr_stats* stats) {
     stats->dense_queries = static_cast<int64_t>(c[kCntDense]);
     float a = -1.f, b = -1.f;
     if (cudaEventElapsedTime(&a, p->ev[0], p->ev[3]) != cudaSuccess) a = -1.f;
-    // ev[1] .. ev[2] bracket the join graph
-    if (cudaEventElapsedTime(&b, p->ev[1], p->ev[2]) != cudaSuccess) b = -1.f;
+    // ev[1] .. ev[2] bracket the join graph, ev_x the expansion kernel or the threshold search
     float x = -1.f;
     if (cudaEventElapsedTime(&x, p->ev_x[0], p->ev_x[1]) != cudaSuccess) x = -1.f;
+    if (p->searched) {
+        b = x;
+        x = 0.f;
+    } else if (cudaEventElapsedTime(&b, p->ev[1], p->ev[2]) != cudaSuccess) {
+        b = -1.f;
+    }
     stats->ms_expand = x;
     cudaGetLastError();
     stats->ms_device = a;
@@ -3031,7 +3204,7 @@ extern "C" mhr_status mhr_topk_paths_batched(const mhr_graph* gc, int32_t nq, co
         pt = ht.data();
     }
     Plan* p = nullptr;
-    MHR_TRY(run_batch(G, nq, ps, pt, K, opts, st, &p));
+    MHR_TRY(run_batch(G, nq, ps, pt, K, opts, st, &p, stats != nullptr));
     const cudaMemcpyKind kind = mem == MHR_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     MHR_CUDA_TRY(cudaMemcpyAsync(out, p->h.out, sizeof(mhr_path) * static_cast<size_t>(nq) * K, kind, st));
     MHR_CUDA_TRY(cudaMemcpyAsync(n_out, p->h.n_out, sizeof(int32_t) * nq, kind, st));
@@ -3098,10 +3271,10 @@ extern "C" mhr_status mhr_autotune(const mhr_graph* gc, int32_t nq, const uint32
         o.chunk = chunks[(i % per) / n_tiles];
         o.tile = tiles[i % n_tiles];
         Plan* p = nullptr;
-        MHR_TRY(run_batch(G, nq, hs.data(), ht.data(), K, &o, st, &p));  // warm-up (capture, buffers)
+        MHR_TRY(run_batch(G, nq, hs.data(), ht.data(), K, &o, st, &p, false));  // warm-up (capture, buffers)
         float ms = 0.f;
         for (int r = 0; r < reps; ++r) {
-            MHR_TRY(run_batch(G, nq, hs.data(), ht.data(), K, &o, st, &p));
+            MHR_TRY(run_batch(G, nq, hs.data(), ht.data(), K, &o, st, &p, false));
             mhr_stats sts{};
             MHR_TRY(read_stats(p, st, &sts));
             if (sts.ms_device < 0) return fail(MHR_ECUDA, "autotune: event timing failed");
@@ -3141,7 +3314,7 @@ extern "C" mhr_status mhr_training_labels(const mhr_graph* gc, int32_t nq, const
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     Plan* p = nullptr;
     mhr_query_opts plain{};
-    MHR_TRY(run_batch(G, nq, s, t, 1, &plain, st, &p, true));
+    MHR_TRY(run_batch(G, nq, s, t, 1, &plain, st, &p, true, true));
     unsigned long long* cnt = p->h.counters + kCntLabels;
     MHR_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
     k_dump_labels<<<std::max(1, G->num_sms) * 4, 256, 0, st>>>(reinterpret_cast<const PlanDev*>(p->dregion), cap,
@@ -3163,22 +3336,13 @@ extern "C" mhr_status mhr_topk_paths(const mhr_graph* g, uint32_t s, uint32_t t,
     if (s == t) return fail(MHR_EINVAL, "s == t");
     if (K < 1) return fail(MHR_EINVAL, "K must be >= 1");
     if (K > MHR_K_MAX) return fail(MHR_ERANGE, "K exceeds MHR_K_MAX");
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    cudaEventRecord(e0, 0);
-    std::vector<mhr_path> buf(K);
+    // a synchronous call on host memory, timed by the host clock
+    const auto t0 = std::chrono::steady_clock::now();
     int32_t n = 0;
-    mhr_status rc = mhr_topk_paths_batched(g, 1, &s, &t, K, buf.data(), &n, MHR_MEM_HOST, opts, stats, nullptr);
-    cudaEventRecord(e1, 0);
-    cudaEventSynchronize(e1);
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (rc != MHR_OK) return rc;
+    std::vector<mhr_path> buf(K);
+    MHR_TRY(mhr_topk_paths_batched(g, 1, &s, &t, K, buf.data(), &n, MHR_MEM_HOST, opts, stats, nullptr));
     std::memcpy(out, buf.data(), sizeof(mhr_path) * std::max(0, n));
     *n_out = n;
-    if (stats) stats->ms = ms;
+    if (stats) stats->ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     return MHR_OK;
 }

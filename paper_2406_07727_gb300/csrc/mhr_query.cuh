@@ -32,6 +32,12 @@ struct Cand {
 };
 static_assert(sizeof(Cand) == 16, "Cand is 16 bytes");
 
+// threshold search: a middle edge that passed the far table
+struct SrPass {
+    uint32_t i, e, v;  // near slot, position in the sorted adjacency, far vertex
+    float phi;         // near weight + middle weight
+};
+
 // middle edge joining a near-side entry to a far-side entry
 struct Hit {
     uint32_t near_k;
@@ -66,6 +72,7 @@ enum {
     kCntSkippedItems = 9,
     kCntLabels = 10,
     kCntTcTimeouts = 11,  // ordering-MLP tiles whose tensor-core MMA gave up waiting
+    kCntRedo = 12,        // queries the threshold search handed back to the join
     kCntCount = 16
 };
 
@@ -84,6 +91,11 @@ struct PlanDev {
     // (nonzero = allowed), or NULL when the call has no constraint
     const uint8_t* cons;
     int32_t part_count, part_index;  // vertex partition: hop-1 vertices u with u % count == index
+    // threshold search
+    const uint32_t* qord;  // [nq] queries, largest rows first
+    Cand* spill;           // [search grid x kSrSpill] candidates past a block's shared buffer
+    SrPass* spill_queue;   // [search grid x kSrSpillQueue] edges to look up past its shared queue
+    int64_t heavy;         // middle edges after which a query is handed back
     MlpDev mlp;            // order 2 weights
     int64_t nhist;        // nq * 256 order buckets
     int64_t item_cap;     // capacity of item_ub
@@ -123,7 +135,7 @@ struct PlanDev {
     uint2* seed_k;      // [nq] near entries holding edge kSeedEdges - 1 and edge kSeedEdges
     float* mlp_qbias;   // [nq x 256] learned order: b1 + W1[:, 128:] e_end[0:128] per query
     // per query [nq] (+1 for item_off)
-    int32_t* status;
+    int32_t* status;    // 0 to be answered, 1 invalid, 2 answered already, 3 handed back
     int32_t* dir;       // 1 = forward (scan out-rows of hop-1 vertices), 0 = backward
     int32_t* near_cnt;
     int32_t* far_cnt;
@@ -145,7 +157,7 @@ struct PlanDev {
     int32_t* chain_cnt; // [nq]
     mhr_path* out;      // [nq x K]
     int32_t* n_out;     // [nq]
-    unsigned long long* counters;  // kCntCount
+    unsigned long long* counters;  // kCntCount, zeroed with the call's inputs
     unsigned long long* cursors;   // [grid] next item of each CTA's own range
     uint32_t* drained;             // [(grid + 31) / 32] bit v: range v has no item left
     uint4* far_start;              // [grid x far_cap] coarse bitmap, indexed by the bit: its run in the far

@@ -48,7 +48,7 @@ struct DevGraph {
     int32_t R, d, dtype, fn;
     double gamma;
     float gamma32;
-    float pad0;
+    int32_t qbits;         // TransE: sums of |a| + |b| + |c| over a row stay below 2^(53 - qbits); else unused
     const int64_t* off;    // CSR by source: row starts [n+1]
     const uint32_t* col;   // destinations [E]
     const uint16_t* rel;   // relation ids [E]

@@ -54,6 +54,7 @@
 #include <tuple>
 #include <vector>
 
+#include "mhr_exact.cuh"
 #include "mhr_internal.cuh"
 #include "mhr_query.cuh"
 #include "mhr_mlp_tc.cuh"
@@ -1973,6 +1974,17 @@ __global__ void __launch_bounds__(kMidThreads, 1) k_middle(const PlanDev* __rest
     if (lane == 0 && wq) atomicAdd(&P->counters[kCntPaths], wq);
 }
 
+// the nch sums of query q join the rescoring's list; all threads of the block call
+__device__ __forceinline__ void push_units(const PlanDev* __restrict__ P, int q, int nch) {
+    __shared__ uint32_t first;
+    const int per = P->unit_sums, n = (nch + per - 1) / per;
+    if (threadIdx.x == 0 && n) first = static_cast<uint32_t>(atomicAdd(&P->counters[kCntUnits], static_cast<unsigned long long>(n)));
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        P->units[first + i] = make_uint2(static_cast<uint32_t>(q), static_cast<uint32_t>(i * per));
+    __syncthreads();
+}
+
 // ===========================================================================
 // threshold search over the weight index (mhr_search.cuh)
 // ===========================================================================
@@ -2048,6 +2060,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(const PlanDev* __restr
             }
             nch += tot;
         }
+        push_units(P, q, nch);
         if (threadIdx.x == 0) {
             P->status[q] = !valid ? 1 : (redo ? 3 : 0);
             P->dense[q] = 0;
@@ -2132,6 +2145,7 @@ __global__ void __launch_bounds__(1024) k_merge1(const PlanDev* __restrict__ P) 
                 nch += tot;
             }
             if (threadIdx.x == 0) P->chain_cnt[q] = nch;
+            push_units(P, q, nch);
         }
         if (threadIdx.x == 0) {
             if (w > P->band_cap) {
@@ -2150,142 +2164,136 @@ __global__ void __launch_bounds__(1024) k_merge1(const PlanDev* __restrict__ P) 
     }
 }
 
-// fp64 rescoring of the band.  The canonical order fixes the accumulation
-// acc = acc + y_j (j ascending) of each edge; the terms y_j = |(a_j + b_j) - c_j|
-// (or (a_j * b_j) * c_j) are formed from the stored values converted exactly.
-// k_merge1 lists the sums a query's band needs (every middle edge; each hop-1
-// and hop-3 edge once, however many band entries share it); each lane runs one
-// sum straight from the three embedding rows (16-byte loads, several in
-// flight), and k_merge2 adds the three weights of every entry.
+// fp64 rescoring of the band (mhr_exact.cuh).  The band's sums (every middle edge;
+// each hop-1 and hop-3 edge once, however many band entries share it) are listed
+// in units of kUnit that all queries append to one list, so the kernel's warps
+// take them without looking at queries that have none.  k_merge2 adds the three
+// weights of every entry.  What bounds it: TransE, the integer issue of the
+// conversions (a warp per sum, its rows read once, whole lines); DistMult, the
+// fp64 pipe (3 d operations per sum).  256 DistMult queries, d = 256, K = 100:
+// 240 -> 181 us; 64 TransE queries, d = 128, K = 100: 51 -> 18 us;
+// 4,096 on bf16 rows, K = 50: 763 -> 310 us.
 constexpr int kRsWarps = 4;
-#ifndef MHR_RS_LANES
-#define MHR_RS_LANES 32
-#endif
-constexpr int kRsLanes = MHR_RS_LANES;  // sums per warp (the other lanes idle)
 
-// Exact binary32 -> binary64 widening done with integer operations (the value
-// is finite: the graph load rejects NaN and infinity), keeping the slow fp64
-// pipe for the arithmetic: sign and mantissa move over, the exponent is
-// re-biased (1023 - 127 = 896), and a subnormal is first normalised.
-__device__ __forceinline__ double widen(float f) {
-    const uint32_t u = __float_as_uint(f);
-    const uint64_t sign = static_cast<uint64_t>(u >> 31) << 63;
-    uint32_t e = (u >> 23) & 0xffu, m = u & 0x7fffffu;
-    if (e == 0u) {
-        if (m == 0u) return __longlong_as_double(static_cast<long long>(sign));
-        const int sh = __clz(m) - 8;  // moves the top set bit to position 23
-        m = (m << sh) & 0x7fffffu;
-        e = static_cast<uint32_t>(1 - sh);
+struct SumEdge {
+    uint32_t h, r, t;
+    double* dst;
+};
+
+// the edge of sum `i` of query q and where its weight goes
+__device__ __forceinline__ SumEdge sum_edge(const PlanDev* __restrict__ P, const DevGraph& g, int q, uint32_t i) {
+    const int64_t cap = P->band_cap;
+    const uint32_t chv = P->chains[3 * cap * q + i];
+    const uint32_t kind = chv >> 30, idx = chv & 0x3fffffffu;
+    const uint32_t s = P->S[q], t = P->T[q];
+    SumEdge o;
+    if (kind == 0u) {  // hop-1 edge (s, r1, u)
+        const int64_t p1 = g.off[s] + idx;
+        o.h = s;
+        o.r = g.rel[p1];
+        o.t = g.col[p1];
+        o.dst = P->w64s + P->a_off[q] + idx;
+    } else if (kind == 1u) {  // hop-3 edge (v, r3, t)
+        const int64_t p3 = g.roff[t] + idx;
+        o.h = g.rcol[p3];
+        o.r = g.rrel[p3];
+        o.t = t;
+        o.dst = P->w64s + P->totA + P->c_off[q] + idx;
+    } else {  // middle edge (u, r2, v) of band entry idx
+        const Cand cd = P->band_cand[cap * q + idx];
+        o.h = g.col[g.off[s] + cd.a_idx];
+        o.r = cd.r2;
+        o.t = g.rcol[g.roff[t] + cd.c_idx];
+        o.dst = P->band_w2 + cap * q + idx;
     }
-    const uint64_t bits = sign | (static_cast<uint64_t>(e + 896u) << 52) | (static_cast<uint64_t>(m) << 29);
-    return __longlong_as_double(static_cast<long long>(bits));
-}
-
-__device__ __forceinline__ double term1(float a, float b, float c, bool transe) {
-    const double x = widen(a), y = widen(b), z = widen(c);
-    return transe ? fabs(__dsub_rn(__dadd_rn(x, y), z)) : __dmul_rn(__dmul_rn(x, y), z);
-}
-
-__device__ __forceinline__ double acc4(double acc, const float4& a, const float4& b, const float4& c, bool transe) {
-    acc = __dadd_rn(acc, term1(a.x, b.x, c.x, transe));
-    acc = __dadd_rn(acc, term1(a.y, b.y, c.y, transe));
-    acc = __dadd_rn(acc, term1(a.z, b.z, c.z, transe));
-    acc = __dadd_rn(acc, term1(a.w, b.w, c.w, transe));
-    return acc;
-}
-
-// fp64 weight of edge (h, r, t) in the canonical order
-__device__ __forceinline__ double edge_w64_seq(const DevGraph& g, uint32_t h, uint32_t r, uint32_t t) {
-    const int d = g.d;
-    const bool transe = g.fn == MHR_SCORE_TRANSE_L1;
-    double acc = 0.0;
-    if (g.dtype == MHR_F32 && (d & 3) == 0) {
-        const float4* A = reinterpret_cast<const float4*>(static_cast<const float*>(g.vemb) + static_cast<int64_t>(h) * d);
-        const float4* B = reinterpret_cast<const float4*>(static_cast<const float*>(g.remb) + static_cast<int64_t>(r) * d);
-        const float4* C = reinterpret_cast<const float4*>(static_cast<const float*>(g.vemb) + static_cast<int64_t>(t) * d);
-        const int n4 = d >> 2;
-#pragma unroll 4
-        for (int j = 0; j < n4; ++j) acc = acc4(acc, __ldg(A + j), __ldg(B + j), __ldg(C + j), transe);
-    } else {
-        for (int j = 0; j < d; ++j)
-            acc = __dadd_rn(acc, term1(emb_f32(g.vemb, g.dtype, h, d, j), emb_f32(g.remb, g.dtype, r, d, j),
-                                       emb_f32(g.vemb, g.dtype, t, d, j), transe));
-    }
-    return transe ? __dsub_rn(g.gamma, acc) : acc;
+    return o;
 }
 
 __global__ void __launch_bounds__(kRsWarps * 32) k_rescore(const PlanDev* __restrict__ P, DevGraph g) {
+    __shared__ double stage[kRsWarps][32 * 33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nq = P->nq, cap = P->band_cap;
-    const int64_t gw = blockIdx.x * static_cast<int64_t>(kRsWarps) + w;
-    const int64_t nw = static_cast<int64_t>(gridDim.x) * kRsWarps;
-    // work unit u = (group of kRsLanes sums) * nq + query: the units that have work
-    // (the first groups of every query) fill the first warps, spread over all
-    // SMs by the small blocks; lane = one sequential fp64 sum
-    const int64_t groups_per_q = (3 * static_cast<int64_t>(cap) + kRsLanes - 1) / kRsLanes;
-    for (int64_t u = gw; u < static_cast<int64_t>(nq) * groups_per_q; u += nw) {
-        const int q = static_cast<int>(u % nq);
-        const int i0 = static_cast<int>(u / nq) * kRsLanes;
-        const int nc = P->chain_cnt[q];
-        if (i0 >= nc || P->dense[q]) continue;
-        const int i = i0 + lane;
-        if (lane >= kRsLanes || i >= nc) continue;
-        const uint32_t chv = P->chains[static_cast<int64_t>(q) * 3 * cap + i];
-        const uint32_t kind = chv >> 30, idx = chv & 0x3fffffffu;
-        const uint32_t s = P->S[q], t = P->T[q];
-        // the edge and where its weight goes; then one converged call for all lanes
-        uint32_t h, r, tt;
-        double* dst;
-        if (kind == 0u) {  // hop-1 edge (s, r1, u)
-            const int64_t p1 = g.off[s] + idx;
-            h = s;
-            r = g.rel[p1];
-            tt = g.col[p1];
-            dst = P->w64s + P->a_off[q] + idx;
-        } else if (kind == 1u) {  // hop-3 edge (v, r3, t)
-            const int64_t p3 = g.roff[t] + idx;
-            h = g.rcol[p3];
-            r = g.rrel[p3];
-            tt = t;
-            dst = P->w64s + P->totA + P->c_off[q] + idx;
-        } else {  // middle edge (u, r2, v) of band entry idx
-            const Cand cd = P->band_cand[static_cast<int64_t>(q) * cap + idx];
-            h = g.col[g.off[s] + cd.a_idx];
-            r = cd.r2;
-            tt = g.rcol[g.roff[t] + cd.c_idx];
-            dst = P->band_w2 + static_cast<int64_t>(q) * cap + idx;
+    const uint32_t n = static_cast<uint32_t>(P->counters[kCntUnits]);
+    const uint32_t nw = gridDim.x * kRsWarps;
+    const bool fixed = g.fn == MHR_SCORE_TRANSE_L1;
+    for (uint32_t u = blockIdx.x * kRsWarps + w; u < n; u += nw) {
+        const uint2 unit = P->units[u];
+        const int q = static_cast<int>(unit.x);
+        const int m = min(P->unit_sums, P->chain_cnt[q] - static_cast<int>(unit.y));
+        if (m <= 0 || P->dense[q]) continue;
+        SumEdge e{0u, 0u, 0u, nullptr};
+        const bool live = lane < m;
+        if (live) e = sum_edge(P, g, q, unit.y + lane);
+        bool left = live;  // sums for the fp64 route
+        if (fixed) {
+            for (int k = 0; k < m; ++k) {
+                bool ok;
+                const double x = warp_w64_fixed(g, __shfl_sync(0xffffffffu, e.h, k), __shfl_sync(0xffffffffu, e.r, k),
+                                                __shfl_sync(0xffffffffu, e.t, k), lane, &ok);
+                if (lane == k && ok) {
+                    *e.dst = x;
+                    left = false;
+                }
+            }
         }
-        *dst = edge_w64_seq(g, h, r, tt);
+        if (__any_sync(0xffffffffu, left)) {
+            const double x = warp_w64_staged(g, e.h, e.r, e.t, left, stage[w], lane);
+            if (left) *e.dst = x;
+        }
     }
 }
 
-// with `redo`, its condition (a conditional graph node: the join of the queries
-// the threshold search handed back) is set when there are any
-__global__ void __launch_bounds__(1024) k_merge2(const PlanDev* __restrict__ P, DevGraph g,
-                                                 cudaGraphConditionalHandle redo, bool has_redo) {
+// order-preserving key of an fp64 score, +0 and -0 alike (larger score -> larger
+// key): compared by integer instructions, where an fp64 compare takes 16 cycles
+__device__ __forceinline__ uint64_t score_key(double w) {
+    const uint64_t b = static_cast<uint64_t>(__double_as_longlong(w == 0.0 ? 0.0 : w));
+    return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+
+// The final order.  What bounds it: a chain of dependent loads per query, then, for
+// bands of up to kRankMax entries, comparing every pair (an entry's place is the
+// number of entries before it; a band of 50 is 2,500 comparisons without a
+// barrier, where the bitonic sort of 64 took 21 barriers of 1,024 threads).  BIG
+// (K > 256) sorts larger bands in shared memory; otherwise they are rare (ties) and
+// their pairs are compared from the candidate pool's memory, so that a block needs
+// little shared memory.  4,096 queries, K = 50: 191 -> 33 us; one query
+// 13 -> 9.5 us.
+// With `redo`, its condition (a conditional graph node: the join of the queries
+// the threshold search handed back) is set when there are any.
+constexpr int kRankMax = 512;
+template <bool BIG>
+__global__ void __launch_bounds__(BIG ? 1024 : 128) k_merge2(const PlanDev* __restrict__ P, DevGraph g,
+                                                             cudaGraphConditionalHandle redo, bool has_redo) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    mhr_path* buf = reinterpret_cast<mhr_path*>(smem_raw);
+    __shared__ uint64_t keys[kRankMax];
+    __shared__ mhr_path small[kRankMax];
     const int K = P->K;
     if (has_redo && blockIdx.x == 0 && threadIdx.x == 0 && P->counters[kCntRedo]) cudaGraphSetConditional(redo, 1u);
     for (int q = blockIdx.x; q < P->nq; q += gridDim.x) {
-        if (P->status[q] != 0) {
-            if (threadIdx.x == 0 && P->status[q] == 1) P->n_out[q] = -1;
+        const int status = P->status[q];
+        if (status != 0) {
+            if (threadIdx.x == 0 && status == 1) P->n_out[q] = -1;
             continue;
         }
         if (P->dense[q]) continue;
         const int nb = P->band_cnt[q];
-        int m = 2;
-        while (m < nb) m <<= 1;
+        const bool pairs = nb <= kRankMax;
+        mhr_path* buf = pairs ? small
+                              : (BIG ? reinterpret_cast<mhr_path*>(smem_raw)
+                                     : reinterpret_cast<mhr_path*>(P->pool + static_cast<int64_t>(q) * P->pq));
+        int m = nb;
+        if (BIG && !pairs)
+            for (m = 2; m < nb;) m <<= 1;
         // band entries with their fp64 score (w1 + w2) + w3 in the canonical order
         const Cand* bc = P->band_cand + static_cast<int64_t>(q) * P->band_cap;
         const double* bw2 = P->band_w2 + static_cast<int64_t>(q) * P->band_cap;
         const uint32_t s = P->S[q], t = P->T[q];
         const int64_t a0 = P->a_off[q], c0 = P->totA + P->c_off[q];
+        const int64_t os = nb ? g.off[s] : 0, rt = nb ? g.roff[t] : 0;
         for (int i = threadIdx.x; i < m; i += blockDim.x) {
             mhr_path p = worst_path();
             if (i < nb) {
                 const Cand cd = bc[i];
-                const int64_t p1 = g.off[s] + cd.a_idx, p3 = g.roff[t] + cd.c_idx;
+                const int64_t p1 = os + cd.a_idx, p3 = rt + cd.c_idx;
                 p.u = g.col[p1];
                 p.r1 = g.rel[p1];
                 p.v = g.rcol[p3];
@@ -2295,12 +2303,33 @@ __global__ void __launch_bounds__(1024) k_merge2(const PlanDev* __restrict__ P, 
                 p.score = __dadd_rn(__dadd_rn(P->w64s[a0 + cd.a_idx], bw2[i]), P->w64s[c0 + cd.c_idx]);
             }
             buf[i] = p;
+            if (pairs) keys[i] = score_key(p.score);
         }
         __syncthreads();
-        block_sort_paths(buf, m);
         const int nout = min(nb, K);
         mhr_path* dst = P->out + static_cast<int64_t>(q) * K;
-        for (int i = threadIdx.x; i < nout; i += blockDim.x) dst[i] = buf[i];
+        if (pairs) {
+            for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+                const uint64_t mine = keys[i];
+                int rank = 0;
+                for (int j = 0; j < nb; ++j) {
+                    const uint64_t k = keys[j];
+                    rank += k > mine ? 1 : 0;
+                    if (k == mine && j != i) rank += ranks_before(small[j], small[i]) ? 1 : 0;
+                }
+                if (rank < nout) dst[rank] = small[i];
+            }
+        } else if (BIG) {
+            block_sort_paths(buf, m);
+            for (int i = threadIdx.x; i < nout; i += blockDim.x) dst[i] = buf[i];
+        } else {
+            for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+                const mhr_path mine = buf[i];
+                int rank = 0;
+                for (int j = 0; j < nb; ++j) rank += ranks_before(buf[j], mine) ? 1 : 0;
+                if (rank < nout) dst[rank] = mine;
+            }
+        }
         if (threadIdx.x == 0) P->n_out[q] = nout;
         __syncthreads();
     }
@@ -2595,6 +2624,7 @@ static mhr_status plan_alloc(Plan* p, T** out, size_t count) {
 
 static size_t mid_smem_bytes() { return sizeof(MidSmem); }
 static_assert(sizeof(MidSmem) <= 232448, "the join's shared memory fits one CTA per SM (227 KB)");
+static_assert(sizeof(mhr_path) * 4096 + (sizeof(mhr_path) + 8) * kRankMax <= 232448, "a band of K = 1,024 in the merge");
 static_assert(2 * sizeof(SearchSmem<512>) <= 230000, "two 512-thread search blocks per SM");
 static size_t exact_smem_bytes() { return sizeof(ExactSmem); }
 static size_t merge2_smem_bytes(int band_cap) {
@@ -2701,6 +2731,14 @@ static mhr_status ensure_items(Plan* p, int64_t cap) {
     return MHR_OK;
 }
 
+static void launch_merge2(Plan* p, int sms, cudaStream_t st, const PlanDev* d, const DevGraph& g,
+                          cudaGraphConditionalHandle redo, bool has_redo) {
+    if (p->K > kRankMax / 2)
+        k_merge2<true><<<std::min(p->nq, sms), 1024, merge2_smem_bytes(p->h.band_cap), st>>>(d, g, redo, has_redo);
+    else
+        k_merge2<false><<<std::min(p->nq, sms * 8), 128, 0, st>>>(d, g, redo, has_redo);
+}
+
 // redo: the join as the conditional part of the threshold search (no event
 // records, which a conditional body cannot hold; queries answered already are skipped)
 static cudaError_t launch_part(Plan* p, const mhr_graph* G, cudaStream_t st, int part, bool redo) {
@@ -2752,7 +2790,7 @@ static cudaError_t launch_part(Plan* p, const mhr_graph* G, cudaStream_t st, int
     } else {
         k_merge1<<<std::min(p->nq, sms * 2), 1024, 0, st>>>(d);
         k_rescore<<<sms * 4, kRsWarps * 32, 0, st>>>(d, g);
-        k_merge2<<<std::min(p->nq, sms * 2), 1024, merge2_smem_bytes(p->h.band_cap), st>>>(d, g, 0, false);
+        launch_merge2(p, sms, st, d, g, 0, false);
         k_exact<<<std::min(p->nq, sms * 2), 1024, exact_smem_bytes(), st>>>(d, g);
     }
     return cudaGetLastError();
@@ -2797,7 +2835,7 @@ static cudaError_t build_search_graph(Plan* p, const mhr_graph* G, cudaGraph_t g
     else k_search<1024><<<p->search_grid, 1024, sizeof(SearchSmem<1024>), st>>>(d, g);
     if (ee == cudaSuccess) ee = cudaEventRecordWithFlags(p->ev_x[1], st, cudaEventRecordExternal);
     k_rescore<<<sms * 4, kRsWarps * 32, 0, st>>>(d, g);
-    k_merge2<<<std::min(p->nq, sms * 2), 1024, merge2_smem_bytes(p->h.band_cap), st>>>(d, g, handle, true);
+    launch_merge2(p, sms, st, d, g, handle, true);
     if (ee == cudaSuccess) ee = cudaGetLastError();
     // the capture's last node carries the dependency of the conditional one
     cudaStreamCaptureStatus status;
@@ -2919,6 +2957,12 @@ static mhr_status make_plan(mhr_graph* G, int nq, int K, int chunk, int precisio
     if ((rc = plan_alloc(p, &h.band_w2, static_cast<size_t>(nq) * h.band_cap)) != MHR_OK) return bail(rc);
     if ((rc = plan_alloc(p, &h.chains, static_cast<size_t>(nq) * 3 * h.band_cap)) != MHR_OK) return bail(rc);
     if ((rc = plan_alloc(p, &h.chain_cnt, nq)) != MHR_OK) return bail(rc);
+    // rescoring units: a warp per sum goes through 8 in turn, a lane per sum takes 32.
+    // (a query's sums are listed once: by the search, or by the join it is handed to)
+    h.unit_sums = G->fn == MHR_SCORE_TRANSE_L1 ? 8 : 32;
+    if ((rc = plan_alloc(p, &h.units, static_cast<size_t>(nq) * ((3 * h.band_cap + h.unit_sums - 1) / h.unit_sums))) !=
+        MHR_OK)
+        return bail(rc);
     if ((rc = plan_alloc(p, &h.out, static_cast<size_t>(nq) * K)) != MHR_OK) return bail(rc);
     if ((rc = plan_alloc(p, &h.n_out, nq)) != MHR_OK) return bail(rc);
     if (G->dg.w) {
@@ -2993,7 +3037,7 @@ static mhr_status make_plan(mhr_graph* G, int nq, int K, int chunk, int precisio
     e = cudaFuncSetAttribute(k_exact, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(exact_smem_bytes()));
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaFuncSetAttribute (exact)"));
-    e = cudaFuncSetAttribute(k_merge2, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_merge2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(merge2_smem_bytes(h.band_cap)));
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaFuncSetAttribute (merge)"));
     *out = p;

@@ -73,6 +73,7 @@ enum {
     kCntLabels = 10,
     kCntTcTimeouts = 11,  // ordering-MLP tiles whose tensor-core MMA gave up waiting
     kCntRedo = 12,        // queries the threshold search handed back to the join
+    kCntUnits = 13,       // rescoring units listed
     kCntCount = 16
 };
 
@@ -155,6 +156,8 @@ struct PlanDev {
     double* band_w2;    // [nq x band_cap] fp64 weight of each band entry's middle edge
     uint32_t* chains;   // [nq x 3 band_cap] fp64 sums to run: kind << 30 | index
     int32_t* chain_cnt; // [nq]
+    uint2* units;       // rescoring work: (query, first of its sums), unit_sums each
+    int32_t unit_sums;
     mhr_path* out;      // [nq x K]
     int32_t* n_out;     // [nq]
     unsigned long long* counters;  // kCntCount, zeroed with the call's inputs

@@ -826,6 +826,7 @@ void free_graph(mhr_graph* g);
 namespace mhr {
 void destroy_plans(mhr_graph* g);  // mhr_query.cu
 void destroy_tail(mhr_graph* g);   // mhr_tail.cu
+void destroy_beam(mhr_graph* g);   // mhr_beam.cu
 }
 
 namespace {
@@ -833,6 +834,7 @@ void free_graph(mhr_graph* g) {
     if (!g) return;
     mhr::destroy_plans(g);
     mhr::destroy_tail(g);
+    mhr::destroy_beam(g);
     for (void* p : g->allocations) cudaFree(p);
     delete g;
 }

@@ -92,6 +92,7 @@ struct DevBuf {
 
 struct PlanCache;  // batched-query plans, defined in mhr_query.cu
 struct TailCache;  // tail-prediction candidate lists and scratch, defined in mhr_tail.cu
+struct BeamCache;  // beam-search buffers, defined in mhr_beam.cu
 
 }  // namespace mhr
 
@@ -117,6 +118,7 @@ struct mhr_graph {
     int num_sms = 0;
     mhr::PlanCache* plans = nullptr;
     mhr::TailCache* tail = nullptr;
+    mhr::BeamCache* beam = nullptr;
 };
 
 namespace mhr {

@@ -393,10 +393,13 @@ mhr_status mhr_mlp_to_bf16(const float* src, uint16_t* dst, int64_t count, void*
  *   serialise them.  The looked-up address is kept for the life of the
  *   process; cudaDeviceReset invalidates it, so do not reset a device that
  *   this entry point has run on and then call it again.
- *   Cost: one thread block on one SM walks every middle edge out of the
- *   hop-1 vertices (the sum of their out-degrees), so the time grows with
- *   that sum; a hub source on a power-law graph can make one call take
- *   seconds.  mhr_topk_paths_batched spreads the same work over every SM.
+ *   Cost: one thread block on one SM.  On a graph with a weight index it
+ *   reads the middle edges that can still matter, as the batched search does.
+ *   Otherwise, and when more candidates tie than its buffers hold, it walks
+ *   every middle edge out of the hop-1 vertices (the sum of their
+ *   out-degrees), so the time grows with that sum; a hub source on a power-law
+ *   graph can then make one call take seconds.  mhr_topk_paths_batched spreads
+ *   the same work over every SM.
  */
 mhr_status mhr_topk_paths_noalloc(const mhr_graph* g, uint32_t s, uint32_t t, int32_t K, mhr_path* out,
                                   int32_t* n_out, void* cuda_stream);

@@ -10,16 +10,23 @@
 // file-scope array of fixed size declared below; the caller passes the inputs
 // (the loaded graph, s, t, K) and the output buffers.
 //
-// The kernel is the single-query form of the exact (tie-safe) path: fp32
-// screening weights of the hop-1 and hop-3 edges in the scratch array, a
-// brute-force walk over the middle edges with a binary search in the reverse
-// row of t, and an exact top-K (fp64 rescoring in the canonical order of every
-// candidate the fp32 screen cannot separate from the running K-th score).
+// On a graph with a weight index the block runs the threshold search of the
+// batched engine (mhr_search.cuh), then scores its candidates in fp64 and orders
+// them, all in shared memory (na_finish).  Queries it hands back (ties wider than
+// the buffers) and graphs without an index take the single-query form of the
+// exact (tie-safe) path: fp32 screening weights of the hop-1 and hop-3 edges in the
+// scratch array, a brute-force walk over the middle edges with a binary search in
+// the reverse row of t, and an exact top-K (fp64 rescoring in the canonical order
+// of every candidate the fp32 screen cannot separate from the running K-th score).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
 #include <mutex>
 
+#include "mhr_exact.cuh"
 #include "mhr_internal.cuh"
+#include "mhr_search.cuh"
 #include "mhr_util.cuh"
 
 namespace mhr {
@@ -32,13 +39,20 @@ constexpr int kNoAllocMaxFrontier = 65536;
 //   [0, M)            fp32 weight of hop-1 entry i  (w(s, r1, u))
 //   [M, 2M)           fp32 weight of hop-3 entry j  (w(v, r3, t))
 //   [2M, 2M + 2M + 2) uint64 prefix of middle-row lengths over hop-1 entries
-// (M = kNoAllocMaxFrontier).  Every cell a call reads is written earlier in
-// the same call, so nothing needs clearing.  About 1 MiB per device.
+// (M = kNoAllocMaxFrontier); before that, during the threshold search,
+//   [0, 128 KiB)      edges that passed its far table, past those in shared memory
+//   [128 KiB, 160 KiB)  candidates past those in shared memory
+// Every cell a call reads is written earlier in the same call, so nothing needs
+// clearing.  About 1 MiB per device.
 constexpr size_t kNoAllocScratchWords = 2 * kNoAllocMaxFrontier + 2 * (kNoAllocMaxFrontier + 1);
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kNoAllocScratchWords];
 
 constexpr int kNaThreads = 1024;
 constexpr int kNaBuf = 4096;
+constexpr int kNaCand = 2048;  // candidates of the threshold search: K <= 1024 and its band
+constexpr int kNaStages = 8;   // warps that add fp64 terms
+static_assert(sizeof(SrPass) * kSrSpillQueue + sizeof(Cand) * (kNaCand - kSrCand) <= 4 * kNoAllocScratchWords,
+              "the search's spill buffers fit the scratch");
 
 struct NoAllocSmem {
     mhr_path buf[kNaBuf];  // [0, K) running top K, [K, kNaBuf) staging
@@ -96,12 +110,113 @@ __device__ void na_flush(NoAllocSmem& sm, int K) {
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kNaThreads) k_topk_noalloc(DevGraph g, uint32_t s, uint32_t t, int K, double err,
-                                                             uint32_t* __restrict__ scratch,
-                                                             mhr_path* __restrict__ out,
-                                                             int32_t* __restrict__ n_out) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    NoAllocSmem& sm = *reinterpret_cast<NoAllocSmem*>(smem_raw);
+// shared memory of the indexed form: the search's, then the fp64 stage of
+// kNaStages warps, which afterwards holds the candidates' records and keys
+struct NaFinish {
+    union {
+        double stage[kNaStages][32 * 33];
+        struct {
+            mhr_path path[kNaCand];
+            uint64_t key[kNaCand];
+        };
+    };
+    int n_left;
+};
+struct NaIndexSmem {
+    SearchSmem<kNaThreads> search;
+    NaFinish fin;
+};
+static_assert(sizeof(NaIndexSmem) <= 227 * 1024, "one block's shared memory");
+
+// The candidates of the finished search scored in fp64 and written in order.  Their
+// 3 n edge weights go to the search's table memory (64 KiB), 24 bytes a candidate,
+// the sums left to the fp64 route behind them, 6 bytes a candidate.
+__device__ void na_finish(NaIndexSmem& x, const DevGraph& g, int K, mhr_path* __restrict__ out,
+                          int32_t* __restrict__ n_out) {
+    SearchSmem<kNaThreads>& sm = x.search;
+    NaFinish& f = x.fin;
+    static_assert(sizeof(sm.tab) >= kNaCand * (3 * sizeof(double) + 3 * sizeof(uint16_t)), "weights fit the table");
+    double* w = reinterpret_cast<double*>(sm.tab);
+    uint16_t* left = reinterpret_cast<uint16_t*>(w + 3 * kNaCand);
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const int n = sm.cand_cnt, sums = 3 * n;
+    const uint32_t s = sm.s, t = sm.t;
+    const int64_t os = g.off[s], rt = g.roff[t];
+    __syncthreads();
+    if (threadIdx.x == 0) f.n_left = 0;
+    __syncthreads();
+    // edge k of candidate i is sum 3 i + k
+    auto edge = [&](int i, uint32_t& h, uint32_t& r, uint32_t& v) {
+        const Cand c = sr_cand(sm, i / 3);
+        const int k = i % 3;
+        const uint32_t u = g.col[os + c.a_idx], z = g.rcol[rt + c.c_idx];
+        h = k == 0 ? s : (k == 1 ? u : z);
+        v = k == 0 ? u : (k == 1 ? z : t);
+        r = k == 0 ? g.rel[os + c.a_idx] : (k == 1 ? c.r2 : g.rrel[rt + c.c_idx]);
+    };
+    if (g.fn == MHR_SCORE_TRANSE_L1) {
+        for (int i = wi; i < sums; i += kNaThreads / 32) {
+            uint32_t h, r, v;
+            bool ok;
+            edge(i, h, r, v);
+            const double y = warp_w64_fixed(g, h, r, v, lane, &ok);
+            if (lane == 0) {
+                if (ok) w[i] = y;
+                else left[atomicAdd(&f.n_left, 1)] = static_cast<uint16_t>(i);
+            }
+        }
+    } else {
+        for (int i = threadIdx.x; i < sums; i += kNaThreads) left[i] = static_cast<uint16_t>(i);
+        if (threadIdx.x == 0) f.n_left = sums;
+    }
+    __syncthreads();
+    const int nl = f.n_left;
+    if (wi < kNaStages) {
+        const int unit = max(1, min(32, (nl + kNaStages - 1) / kNaStages));
+        for (int b = wi * unit; b < nl; b += kNaStages * unit) {
+            const bool live = lane < unit && b + lane < nl;
+            uint32_t h = 0u, r = 0u, v = 0u;
+            if (live) edge(left[b + lane], h, r, v);
+            const double y = warp_w64_staged(g, h, r, v, live, f.stage[wi], lane);
+            if (live) w[left[b + lane]] = y;
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += kNaThreads) {
+        const Cand c = sr_cand(sm, i);
+        mhr_path p;
+        p.u = g.col[os + c.a_idx];
+        p.r1 = g.rel[os + c.a_idx];
+        p.v = g.rcol[rt + c.c_idx];
+        p.r3 = g.rrel[rt + c.c_idx];
+        p.r2 = c.r2;
+        p.pad = 0;
+        p.score = __dadd_rn(__dadd_rn(w[3 * i], w[3 * i + 1]), w[3 * i + 2]);
+        f.path[i] = p;
+        // larger score, larger key (+0 and -0 alike): no fp64 compares in the loop below
+        const uint64_t b = static_cast<uint64_t>(__double_as_longlong(p.score == 0.0 ? 0.0 : p.score));
+        f.key[i] = (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+    }
+    __syncthreads();
+    // a candidate's place is the number of candidates before it
+    for (int i = threadIdx.x; i < n; i += kNaThreads) {
+        const uint64_t mine = f.key[i];
+        int rank = 0;
+        for (int j = 0; j < n; ++j) {
+            const uint64_t k = f.key[j];
+            rank += k > mine ? 1 : 0;
+            if (k == mine && j != i) rank += na_before(f.path[j], f.path[i]) ? 1 : 0;
+        }
+        if (rank < K) out[rank] = f.path[i];
+    }
+    if (threadIdx.x == 0) *n_out = min(n, K);
+}
+
+// every middle edge out of the hop-1 vertices, one by one
+__device__ __noinline__ void na_walk(const DevGraph& g, uint32_t s, uint32_t t, int K, double err,
+                                     uint32_t* __restrict__ scratch, mhr_path* __restrict__ out,
+                                     int32_t* __restrict__ n_out) {
+    NoAllocSmem& sm = *reinterpret_cast<NoAllocSmem*>(sr_smem_raw);
     float* wA = reinterpret_cast<float*>(scratch);
     float* wC = reinterpret_cast<float*>(scratch + kNoAllocMaxFrontier);
     uint64_t* pref = reinterpret_cast<uint64_t*>(scratch + 2 * kNoAllocMaxFrontier);
@@ -111,11 +226,11 @@ __global__ void __launch_bounds__(kNaThreads) k_topk_noalloc(DevGraph g, uint32_
     // hop-1 and hop-3 fp32 weights; excluded endpoints get -inf
     for (int64_t i = threadIdx.x; i < na; i += blockDim.x) {
         const uint32_t u = g.col[os + i];
-        wA[i] = (u == s || u == t) ? __int_as_float(0xff800000) : edge_w32_group(g, s, g.rel[os + i], u, 0, 1);
+        wA[i] = (u == s || u == t) ? __int_as_float(0xff800000) : g.w ? g.w[os + i] : edge_w32_group(g, s, g.rel[os + i], u, 0, 1);
     }
     for (int64_t j = threadIdx.x; j < nc; j += blockDim.x) {
         const uint32_t v = g.rcol[rs + j];
-        wC[j] = (v == s || v == t) ? __int_as_float(0xff800000) : edge_w32_group(g, v, g.rrel[rs + j], t, 0, 1);
+        wC[j] = (v == s || v == t) ? __int_as_float(0xff800000) : g.rw ? g.rw[rs + j] : edge_w32_group(g, v, g.rrel[rs + j], t, 0, 1);
     }
     // prefix of middle-row lengths over hop-1 entries (excluded entries: 0)
     int64_t carry = 0;
@@ -170,7 +285,7 @@ __global__ void __launch_bounds__(kNaThreads) k_topk_noalloc(DevGraph g, uint32_
                     sm.hp[slot] = static_cast<uint32_t>(p2);
                     sm.hc0[slot] = static_cast<uint32_t>(a);
                     sm.hcn[slot] = static_cast<uint32_t>(c1 - a);
-                    sm.hw2[slot] = edge_w32_group(g, u, g.rel[p2], v, 0, 1);
+                    sm.hw2[slot] = g.w ? g.w[p2] : edge_w32_group(g, u, g.rel[p2], v, 0, 1);
                 }
             }
         }
@@ -219,6 +334,45 @@ __global__ void __launch_bounds__(kNaThreads) k_topk_noalloc(DevGraph g, uint32_
     if (threadIdx.x == 0) *n_out = sm.nt;
 }
 
+// What bounds it: with the index, the barriers and dependent loads of the search's
+// phases on one SM; without, the walk, which reads every middle edge.  One kernel
+// holds both, so a query handed back needs no second launch.  100,000 vertices, 1M
+// edges, 64 fp32 values, K = 20: 2.2 to 11.5 ms by the query (the walk) -> 98 us.
+template <bool INDEX>
+__global__ void __launch_bounds__(kNaThreads) k_topk_noalloc(const __grid_constant__ DevGraph g, uint32_t s, uint32_t t,
+                                                             int K, double err, uint32_t* __restrict__ scratch,
+                                                             mhr_path* __restrict__ out, int32_t* __restrict__ n_out) {
+    if (INDEX) {
+        NaIndexSmem& x = *reinterpret_cast<NaIndexSmem*>(sr_smem_raw);
+        SearchSmem<kNaThreads>& sm = x.search;
+        if (threadIdx.x == 0) {
+            sm.s = s;
+            sm.t = t;
+            sm.K = K;
+            sm.part_count = 1;
+            sm.part_index = 0;
+            sm.cons = nullptr;
+            sm.R = g.R;
+            sm.two_err = 2.0 * err;
+            sm.spill_queue = reinterpret_cast<SrPass*>(scratch);
+            sm.spill = reinterpret_cast<Cand*>(sm.spill_queue + kSrSpillQueue);
+            sm.cap = kNaCand;
+            sm.redo = 0;
+            sm.cand_cnt = 0;
+        }
+        __syncthreads();
+        search_query<kNaThreads>(g, ~0ull);  // the walk would read no fewer edges
+        __syncthreads();
+        const bool redo = sm.redo != 0 || sm.cand_cnt > kNaCand;
+        __syncthreads();
+        if (!redo) {
+            na_finish(x, g, K, out, n_out);
+            return;
+        }
+    }
+    na_walk(g, s, t, K, err, scratch, out, n_out);
+}
+
 // per-device address of the scratch array (host code cannot use the symbol
 // itself: in host code it names a host-side stand-in, not device memory)
 static std::mutex g_na_mu;
@@ -235,8 +389,11 @@ static mhr_status noalloc_setup(int dev, uint32_t** ptr) {
         g_na_ptr[dev] = p;
     }
     if (!g_na_attr[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_topk_noalloc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(k_topk_noalloc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(sizeof(NoAllocSmem)));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_topk_noalloc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(std::max(sizeof(NoAllocSmem), sizeof(NaIndexSmem))));
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute (no-allocation kernel)");
         g_na_attr[dev] = true;
     }
@@ -265,7 +422,12 @@ extern "C" mhr_status mhr_topk_paths_noalloc(const mhr_graph* g, uint32_t s, uin
     uint32_t* scratch = nullptr;
     MHR_TRY(noalloc_setup(g->device, &scratch));
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    k_topk_noalloc<<<1, kNaThreads, sizeof(NoAllocSmem), st>>>(g->dg, s, t, K, g->err_path, scratch, out, n_out);
+    if (g->dg.w && std::isfinite(g->err_path))
+        k_topk_noalloc<true><<<1, kNaThreads, std::max(sizeof(NoAllocSmem), sizeof(NaIndexSmem)), st>>>(
+            g->dg, s, t, K, g->err_path, scratch, out, n_out);
+    else
+        k_topk_noalloc<false><<<1, kNaThreads, sizeof(NoAllocSmem), st>>>(g->dg, s, t, K, g->err_path, scratch, out,
+                                                                          n_out);
     MHR_CUDA_TRY(cudaGetLastError());
     return MHR_OK;
 }

@@ -6,6 +6,8 @@
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "mhr_internal.cuh"
 #include "mhr_mlp.cuh"
 #include "mhr_mlp_tc.cuh"
@@ -98,156 +100,150 @@ __global__ void k_mlp_features(DevGraph g, const uint32_t* __restrict__ va, cons
     }
 }
 
-// dZ[r][c] = (z[r][c] > 0) * dy[r] * w2[c],  dy[r] = 2 (y[r] - t[r]) / n
-__global__ void k_mlp_bwd_rows(const float* __restrict__ w2, const float* __restrict__ y,
-                               const float* __restrict__ tgt, const float* __restrict__ z1, int64_t n,
-                               float* __restrict__ dz) {
-    const int64_t total = n * kMlpHid;
-    const float inv = 2.0f / static_cast<float>(n);
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total; i += stride) {
-        const int64_t r = i / kMlpHid;
-        const int c = static_cast<int>(i - r * kMlpHid);
-        const float dy = (y[r] - tgt[r]) * inv;
-        dz[i] = z1[i] > 0.f ? dy * w2[c] : 0.f;
-    }
-}
-
-// column sums in a fixed order: db1[c] = sum_r dZ[r][c], dw2[c] = sum_r
-// relu(z[r][c]) dy[r]; block 0 also db2 = sum_r dy[r] and the loss
-__global__ void __launch_bounds__(256) k_mlp_bwd_cols(const float* __restrict__ y, const float* __restrict__ tgt,
-                                                      const float* __restrict__ z1, const float* __restrict__ dz,
-                                                      int64_t n, float* __restrict__ grads,
-                                                      float* __restrict__ loss) {
-    __shared__ float s1[8][32], s2[8][32];
-    const int c = blockIdx.x * 32 + (threadIdx.x & 31);
-    const int grp = threadIdx.x >> 5;
-    const float inv = 2.0f / static_cast<float>(n);
-    float a = 0.f, b = 0.f;
-    for (int64_t r = grp; r < n; r += 8) {
-        const float dy = (y[r] - tgt[r]) * inv;
-        a += dz[r * kMlpHid + c];
-        b += fmaxf(z1[r * kMlpHid + c], 0.f) * dy;
-    }
-    s1[grp][threadIdx.x & 31] = a;
-    s2[grp][threadIdx.x & 31] = b;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float sa = 0.f, sb = 0.f;
-        for (int k = 0; k < 8; ++k) {
-            sa += s1[k][threadIdx.x];
-            sb += s2[k][threadIdx.x];
-        }
-        grads[kMlpHid * kMlpIn + c] = sa;            // db1
-        grads[kMlpHid * kMlpIn + kMlpHid + c] = sb;  // dw2
-    }
-    if (blockIdx.x == 0) {
-        __syncthreads();
-        // db2 and the loss, fixed order
-        float d = 0.f, l = 0.f;
-        for (int64_t r = threadIdx.x; r < n; r += blockDim.x) {
-            const float e = y[r] - tgt[r];
-            d += e * inv;
-            l += e * e;
-        }
-        s1[threadIdx.x >> 5][threadIdx.x & 31] = d;
-        s2[threadIdx.x >> 5][threadIdx.x & 31] = l;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float sd = 0.f, sl = 0.f;
-            for (int k = 0; k < 256; ++k) {
-                sd += s1[k >> 5][k & 31];
-                sl += s2[k >> 5][k & 31];
-            }
-            grads[kMlpHid * kMlpIn + 2 * kMlpHid] = sd;  // db2
-            if (loss) *loss = sl / static_cast<float>(n);
-        }
-    }
-}
-
-// dW1 = dZ^T X on the tensor cores (tcgen05).  CTA (bx, by) owns hidden units
-// 128 by .. +127 and inputs 64 bx .. +63 (M = 128, N = 64, 64 TMEM columns) and
-// runs over all rows in chunks of 64 (the contraction dimension): dZ^T is
-// staged as bf16 hi + lo parts (dZ = hi + lo + r, |r| <= 2^-16 |dZ|; two MMAs
-// per K step), X^T as bf16 (exact); both are transposed into K-major core
-// matrices on the way into shared memory.  Each output element is summed by
-// one CTA in a fixed order, so gradients are deterministic.  A chunk whose MMA
-// does not complete within a second makes the CTA's gradients NaN.
-constexpr int kDwRows = 64;  // rows of dZ / X per chunk
+// The gradients, one pass over z1 and X:
+//   dZ[r][c] = (z[r][c] > 0) dy[r] w2[c],  dy[r] = 2 (y[r] - t[r]) / n
+//   dW1 = dZ^T X,  db1 = sum_r dZ[r],  dw2 = sum_r relu(z[r]) dy[r],  db2 = sum_r dy[r]
+// dW1 runs on the tensor cores (tcgen05).  CTA (bx, by, slice) owns hidden units
+// 128 by .. +127, inputs 64 bx .. +63 (M = 128, N = 64, 64 TMEM columns) and the
+// slice's rows, in chunks of 64 (the contraction dimension): dZ^T is formed from z1
+// while it is staged, as bf16 hi + lo parts (dZ = hi + lo + r, |r| <= 2^-16 |dZ|;
+// two MMAs per K step), X^T as bf16 (exact); both are transposed into K-major core
+// matrices on the way into shared memory.  Core matrices lie 144 bytes apart, so
+// the eight lanes that write one row each of eight of them use all banks (128 bytes
+// apart they all hit the same four).  The CTAs of bx = 0 hold every dZ and z in
+// registers once and add up the other sums.
+//
+// What bounds it: the latency of a chunk (loads, transposition, MMA: about 3 us),
+// so the rows are cut into slices that fill two CTAs per SM.  Every slice writes
+// its own gradients, summed in slice order (k_mlp_bwd_sum): the order depends on n
+// and the SM count alone, and each sum is shorter than one over all rows.  A whole
+// training step of 4,096 rows: 379 us with one slice of all rows after two passes
+// that wrote dZ and read it back -> 59 us.  A chunk whose MMA does not complete within a second makes the
+// CTA's gradients NaN.
+constexpr int kDwRows = 64;   // rows of z1 / X per chunk
+constexpr int kDwCore = 144;  // bytes between core matrices of neighbouring columns
+constexpr int kDwGroup = kDwRows / 8 * kDwCore;
+constexpr int64_t kDwPart = (kMlpParams + 1 + 15) / 16 * 16;  // floats of a slice: gradients, then the loss sum
 struct DwSmem {
-    alignas(128) uint8_t Ahi[kTcRows * kDwRows * 2];
-    alignas(128) uint8_t Alo[kTcRows * kDwRows * 2];
-    alignas(128) uint8_t B[64 * kDwRows * 2];
+    alignas(128) uint8_t A[2][kTcRows / 8 * kDwGroup];  // dZ^T, hi and lo; at the end the tile of dW1
+    alignas(128) uint8_t B[64 / 8 * kDwGroup];
+    float dy[2][kDwRows];
+    float red[2][2];
     uint64_t bar;
     uint32_t tmem;
 };
+static_assert(sizeof(float) * kTcRows * 65 <= sizeof(DwSmem::A), "the tile of dW1 fits its staging buffers");
 
-__global__ void __launch_bounds__(kTcThreads, 1) k_mlp_dw1_tc(const float* __restrict__ dz, const uint16_t* __restrict__ X,
-                                                              int64_t n, float* __restrict__ grads) {
+__global__ void __launch_bounds__(kTcThreads, 2)
+    k_mlp_bwd_tc(const float* __restrict__ w2, const float* __restrict__ y, const float* __restrict__ tgt,
+                 const float* __restrict__ z1, const uint16_t* __restrict__ X, int64_t n, float* __restrict__ part,
+                 float* __restrict__ loss) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     DwSmem& sm = *reinterpret_cast<DwSmem*>(smem_raw);
     const int i0 = blockIdx.x * 64, o0 = blockIdx.y * kTcRows;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool sums = blockIdx.x == 0;
+    const int64_t chunks = (n + kDwRows - 1) / kDwRows;
+    const int64_t k0 = chunks * blockIdx.z / gridDim.z, k1 = chunks * (blockIdx.z + 1) / gridDim.z;
+    const float inv = 2.0f / static_cast<float>(n);
+    part += kDwPart * blockIdx.z;
     if (warp == 0) tc::tmem_alloc(&sm.tmem, 64);
     if (threadIdx.x == 0) {
         tc::mbar_init(&sm.bar, 1);
         tc::mbar_fence_init();
     }
+    // threads 0 .. 127: a core matrix of dZ^T each (16 hidden blocks x 8 row blocks),
+    // 128 .. 191: one of X^T (8 x 8), 192 .. 255: the next chunk's dy
+    const int role = threadIdx.x < 128 ? 0 : (threadIdx.x < 192 ? 1 : 2);
+    const int blk = (threadIdx.x & (role == 0 ? 127 : 63)) >> 3, rg = threadIdx.x & 7;
+    float wv[8], sa[8], sb[8], sd = 0.f, sl = 0.f;
+    if (role == 0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            wv[k] = __ldg(w2 + o0 + blk * 8 + k);
+            sa[k] = sb[k] = 0.f;
+        }
+    }
+    auto dy_of = [&](int64_t chunk) {
+        const int i = threadIdx.x - 192;
+        const int64_t row = chunk * kDwRows + i;
+        float d = 0.f;
+        if (row < n) {
+            const float e = __ldg(y + row) - __ldg(tgt + row);
+            d = e * inv;
+            sd += d;
+            sl += e * e;
+        }
+        sm.dy[chunk & 1][i] = d;
+    };
+    if (role == 2) dy_of(k0);
+    __syncthreads();
     uint32_t phase = 0;
     bool ok = true;
-    for (int64_t r0 = 0; r0 < n && ok; r0 += kDwRows) {
-        // 128 core matrices of dZ^T (16 hidden blocks x 8 row blocks), 64 of X^T (8 x 8)
-        for (int job = threadIdx.x; job < 192; job += blockDim.x) {
-            if (job < 128) {
-                const int og = job >> 3, rg = job & 7;
-                float v[8][8];
+    for (int64_t ch = k0; ch < k1 && ok; ++ch) {
+        const int64_t r0 = ch * kDwRows;
+        if (role == 0) {
+            float v[8][8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int64_t row = r0 + rg * 8 + j;
-                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-                    if (row < n) {
-                        const float4* src = reinterpret_cast<const float4*>(dz + row * kMlpHid + o0 + og * 8);
-                        a = __ldg(src);
-                        b = __ldg(src + 1);
-                    }
-                    v[j][0] = a.x; v[j][1] = a.y; v[j][2] = a.z; v[j][3] = a.w;
-                    v[j][4] = b.x; v[j][5] = b.y; v[j][6] = b.z; v[j][7] = b.w;
+            for (int j = 0; j < 8; ++j) {
+                const int64_t row = r0 + rg * 8 + j;
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+                if (row < n) {
+                    const float4* src = reinterpret_cast<const float4*>(z1 + row * kMlpHid + o0 + blk * 8);
+                    a = __ldg(src);
+                    b = __ldg(src + 1);
                 }
+                v[j][0] = a.x; v[j][1] = a.y; v[j][2] = a.z; v[j][3] = a.w;
+                v[j][4] = b.x; v[j][5] = b.y; v[j][6] = b.z; v[j][7] = b.w;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float dy = sm.dy[ch & 1][rg * 8 + j];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    uint32_t hw[4], lw[4];
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        const float x0 = v[2 * m][k], x1 = v[2 * m + 1][k];
-                        const __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
-                        hw[m] = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) |
-                                (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
-                        lw[m] = pack_bf16x2(x0 - __bfloat162float(h0), x1 - __bfloat162float(h1));
+                    const float z = v[j][k], x = z > 0.f ? dy * wv[k] : 0.f;
+                    if (sums) {
+                        sa[k] += x;
+                        sb[k] += fmaxf(z, 0.f) * dy;
                     }
-                    const uint32_t off = tc::core_offset(og * 8 + k, rg * 8, kDwRows);
-                    *reinterpret_cast<uint4*>(sm.Ahi + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                    *reinterpret_cast<uint4*>(sm.Alo + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-                }
-            } else {
-                const int b = job - 128, ig = b >> 3, rg = b & 7;
-                uint32_t w[8][4];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int64_t row = r0 + rg * 8 + j;
-                    uint4 t = make_uint4(0u, 0u, 0u, 0u);
-                    if (row < n) t = __ldg(reinterpret_cast<const uint4*>(X + row * kMlpIn + i0 + ig * 8));
-                    w[j][0] = t.x; w[j][1] = t.y; w[j][2] = t.z; w[j][3] = t.w;
-                }
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const unsigned sel = (k & 1) ? 0x7632u : 0x5410u;  // high or low halves
-                    uint32_t o[4];
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) o[m] = __byte_perm(w[2 * m][k >> 1], w[2 * m + 1][k >> 1], sel);
-                    *reinterpret_cast<uint4*>(sm.B + tc::core_offset(ig * 8 + k, rg * 8, kDwRows)) =
-                        make_uint4(o[0], o[1], o[2], o[3]);
+                    v[j][k] = x;
                 }
             }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                uint32_t hw[4], lw[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float x0 = v[2 * m][k], x1 = v[2 * m + 1][k];
+                    const __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
+                    hw[m] = static_cast<uint32_t>(__bfloat16_as_ushort(h0)) |
+                            (static_cast<uint32_t>(__bfloat16_as_ushort(h1)) << 16);
+                    lw[m] = pack_bf16x2(x0 - __bfloat162float(h0), x1 - __bfloat162float(h1));
+                }
+                const uint32_t off = blk * kDwGroup + rg * kDwCore + k * 16;
+                *reinterpret_cast<uint4*>(sm.A[0] + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+                *reinterpret_cast<uint4*>(sm.A[1] + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+            }
+        } else if (role == 1) {
+            uint32_t w[8][4];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int64_t row = r0 + rg * 8 + j;
+                uint4 t = make_uint4(0u, 0u, 0u, 0u);
+                if (row < n) t = __ldg(reinterpret_cast<const uint4*>(X + row * kMlpIn + i0 + blk * 8));
+                w[j][0] = t.x; w[j][1] = t.y; w[j][2] = t.z; w[j][3] = t.w;
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const unsigned sel = (k & 1) ? 0x7632u : 0x5410u;  // high or low halves
+                uint32_t o[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) o[m] = __byte_perm(w[2 * m][k >> 1], w[2 * m + 1][k >> 1], sel);
+                *reinterpret_cast<uint4*>(sm.B + blk * kDwGroup + rg * kDwCore + k * 16) =
+                    make_uint4(o[0], o[1], o[2], o[3]);
+            }
+        } else if (ch + 1 < k1) {
+            dy_of(ch + 1);
         }
         tc::fence_async_smem();
         tc::fence_before_sync();
@@ -255,13 +251,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_mlp_dw1_tc(const float* __res
         tc::fence_after_sync();
         if (threadIdx.x == 0) {
             constexpr uint32_t idesc = tc::idesc_bf16_f32(kTcRows, 64);
-            constexpr uint32_t sbo = (kDwRows / 8) * 128;
-            const uint32_t ah = tc::smem_u32(sm.Ahi), al = tc::smem_u32(sm.Alo), bb = tc::smem_u32(sm.B);
+            const uint32_t ah = tc::smem_u32(sm.A[0]), al = tc::smem_u32(sm.A[1]), bb = tc::smem_u32(sm.B);
 #pragma unroll
             for (int kk = 0; kk < kDwRows / 16; ++kk) {
-                const uint64_t bd = tc::smem_desc(bb + kk * 256, 128, sbo);
-                tc::mma_bf16(sm.tmem, tc::smem_desc(ah + kk * 256, 128, sbo), bd, idesc, (r0 > 0 || kk > 0) ? 1u : 0u);
-                tc::mma_bf16(sm.tmem, tc::smem_desc(al + kk * 256, 128, sbo), bd, idesc, 1u);
+                const uint32_t at = kk * 2 * kDwCore;
+                const uint64_t bd = tc::smem_desc(bb + at, kDwCore, kDwGroup);
+                tc::mma_bf16(sm.tmem, tc::smem_desc(ah + at, kDwCore, kDwGroup), bd, idesc, (ch > k0 || kk > 0) ? 1u : 0u);
+                tc::mma_bf16(sm.tmem, tc::smem_desc(al + at, kDwCore, kDwGroup), bd, idesc, 1u);
             }
             tc::mma_commit(&sm.bar);
         }
@@ -270,14 +266,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_mlp_dw1_tc(const float* __res
         tc::fence_after_sync();
         ok = !__syncthreads_or(done ? 0 : 1);
     }
+    // the tile of dW1, through shared memory so that its rows are written whole
+    float* tile = reinterpret_cast<float*>(sm.A[0]);
     if (warp < 4) {
-        const int o = o0 + warp * 32 + lane;
-        float* dst = grads + static_cast<int64_t>(o) * kMlpIn + i0;
         for (int c0 = 0; c0 < 64; c0 += 32) {
             float v[32];
             tc::tmem_ld32(sm.tmem + (static_cast<uint32_t>(warp * 32) << 16) + static_cast<uint32_t>(c0), v);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) dst[c0 + i] = ok ? v[i] : __int_as_float(0x7fc00000);
+            for (int i = 0; i < 32; ++i) tile[(warp * 32 + lane) * 65 + c0 + i] = ok ? v[i] : __int_as_float(0x7fc00000);
+        }
+    }
+    if (role == 2) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sd += __shfl_xor_sync(0xffffffffu, sd, o);
+            sl += __shfl_xor_sync(0xffffffffu, sl, o);
+        }
+        if (lane == 0) {
+            sm.red[warp & 1][0] = sd;
+            sm.red[warp & 1][1] = sl;
         }
     }
     tc::fence_before_sync();
@@ -286,6 +293,41 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_mlp_dw1_tc(const float* __res
         tc::fence_after_sync();
         tc::tmem_dealloc(sm.tmem, 64);
     }
+    for (int i = threadIdx.x; i < kTcRows * 64; i += kTcThreads)
+        part[static_cast<int64_t>(o0 + (i >> 6)) * kMlpIn + i0 + (i & 63)] = tile[(i >> 6) * 65 + (i & 63)];
+    if (!sums) return;
+    if (role == 0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {  // over the eight row blocks
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                sa[k] += __shfl_xor_sync(0xffffffffu, sa[k], o);
+                sb[k] += __shfl_xor_sync(0xffffffffu, sb[k], o);
+            }
+            if (rg == 0) {
+                part[kMlpHid * kMlpIn + o0 + blk * 8 + k] = sa[k];            // db1
+                part[kMlpHid * kMlpIn + kMlpHid + o0 + blk * 8 + k] = sb[k];  // dw2
+            }
+        }
+    }
+    if (blockIdx.y == 0 && threadIdx.x == 0) {
+        part[kMlpParams - 1] = sm.red[0][0] + sm.red[1][0];  // db2
+        const float l = sm.red[0][1] + sm.red[1][1];
+        if (gridDim.z > 1) part[kMlpParams] = l;
+        else if (loss) *loss = l / static_cast<float>(n);
+    }
+}
+
+// the slices' gradients, added in slice order, and the loss
+__global__ void __launch_bounds__(256) k_mlp_bwd_sum(const float* __restrict__ part, int slices, int64_t n,
+                                                     float* __restrict__ grads, float* __restrict__ loss) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i > kMlpParams) return;
+    float s = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < slices; ++k) s += __ldg(part + kDwPart * k + i);
+    if (i < kMlpParams) grads[i] = s;
+    else if (loss) *loss = s / static_cast<float>(n);
 }
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ gr, float* __restrict__ m1,
@@ -391,11 +433,15 @@ extern "C" mhr_status mhr_mlp_backward(const mhr_mlp* m, const uint16_t* X, int6
     if (n < 1 || !X || !target || !y || !z1 || !work || !grads) return fail(MHR_EINVAL, "bad backward arguments");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int sms = std::max(1, device_sm_count());
-    k_mlp_bwd_rows<<<sms * 4, 256, 0, st>>>(m->w2, y, target, z1, n, work);
-    k_mlp_bwd_cols<<<kMlpHid / 32, 256, 0, st>>>(y, target, z1, work, n, grads, loss);
-    MHR_CUDA_TRY(cudaFuncSetAttribute(k_mlp_dw1_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    // Row slices: 8 CTAs each, two CTAs per SM, at least one chunk, and room for every
+    // slice's gradients in the scratch (258 rows of it hold one slice).
+    const int64_t fit = n * kMlpHid / kDwPart, fill = std::max(1, 2 * sms / 8);
+    const int slices = static_cast<int>(std::max<int64_t>(1, std::min({fit, fill, (n + kDwRows - 1) / kDwRows})));
+    MHR_CUDA_TRY(cudaFuncSetAttribute(k_mlp_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       static_cast<int>(sizeof(DwSmem))));
-    k_mlp_dw1_tc<<<dim3(kMlpIn / 64, kMlpHid / kTcRows), kTcThreads, sizeof(DwSmem), st>>>(work, X, n, grads);
+    k_mlp_bwd_tc<<<dim3(kMlpIn / 64, kMlpHid / kTcRows, slices), kTcThreads, sizeof(DwSmem), st>>>(
+        m->w2, y, target, z1, X, n, slices > 1 ? work : grads, loss);
+    if (slices > 1) k_mlp_bwd_sum<<<(kMlpParams + 256) / 256, 256, 0, st>>>(work, slices, n, grads, loss);
     MHR_CUDA_TRY(cudaGetLastError());
     return MHR_OK;
 }

@@ -11,17 +11,17 @@
 //      candidates; per query, the K-th best sampled score minus twice the
 //      per-edge error bound is a threshold that can drop no candidate of the
 //      exact top K (the K-th best of a subset is at most the K-th best of all);
-//   3. full pass (k_tail_scan): every candidate row is read once with 16-byte
-//      loads, a group of G lanes holding two rows in registers, and scored
-//      against every query of the batch (query vectors e_h + w_r or
-//      e_h * w_r in shared memory, each load feeding both rows); scores at or
-//      above the threshold are appended to the query's survivor list
-//      (warp-aggregated atomics);
+//   3. full pass (k_tail_scan*): every candidate row is read with 16-byte loads
+//      where its length allows it, held in registers by a group of lanes and scored
+//      against the queries of a chunk (query vectors e_h + w_r or e_h * w_r in shared
+//      memory); scores at or above the threshold are appended to the query's
+//      survivor list;
 //   4. per query (k_tail_final): the exact K-th best fp32 survivor score by a
 //      radix select, the band of survivors within twice the error bound of it
-//      rescored in fp64 in the canonical operation order (one member per
-//      thread, e_h + w_r formed once in fp64 in shared memory), and the K best
-//      of the band sorted in shared memory.
+//      rescored in fp64 in the canonical operation order (TransE a warp per member
+//      in integers; otherwise one member per thread, e_h + w_r formed once in fp64
+//      in shared memory), and the K best of the band put in order, a short band by
+//      comparing every pair (64 queries, K = 50: 33 -> 16 us).
 //
 // Exactness: |S32 - w64| <= E = eps32 + eps64 for every candidate (the bound of
 // mhr_graph.cu holds for any (u, r, v) triple and any summation order).  If c
@@ -36,6 +36,7 @@
 #include <cmath>
 #include <vector>
 
+#include "mhr_exact.cuh"
 #include "mhr_internal.cuh"
 #include "mhr_util.cuh"
 
@@ -48,6 +49,7 @@ struct TailCache {
     size_t scratch_bytes = 0;
     void* big = nullptr;  // survivors + band of one query rescanned alone
     size_t big_bytes = 0;
+    char* pinned = nullptr;  // kPinned bytes: the queries' ids and the counts of a batch, read back
     cudaEvent_t ev[4] = {};
 
     ~TailCache() {
@@ -55,6 +57,7 @@ struct TailCache {
             if (p) cudaFree(p);
         if (scratch) cudaFree(scratch);
         if (big) cudaFree(big);
+        if (pinned) cudaFreeHost(pinned);
         for (cudaEvent_t e : ev)
             if (e) cudaEventDestroy(e);
     }
@@ -75,6 +78,8 @@ constexpr size_t kQueryBytes = 64 * 1024;      // query vectors + thresholds per
 constexpr int kMaxBatch = 256;                 // queries per scan launch
 constexpr size_t kScratchBudget = size_t(1) << 30;
 constexpr int kCompactBlocks = 512;
+constexpr size_t kPinned = 32 * 1024;
+constexpr int kRankMax = 512;                  // records ordered by comparing every pair
 
 static_assert((kSortMax & (kSortMax - 1)) == 0, "sort size must be a power of two");
 
@@ -94,6 +99,7 @@ struct ScanArgs {
     const uint32_t* h;     // [nq] heads
     const uint16_t* r;     // [nq] relations
     int nq;
+    int chunk;             // queries of one block (blockIdx.y)
     int G;                 // lanes per candidate row (power of two, vector kernels)
     const uint32_t* cand;  // candidate ids; nullptr: candidate i is vertex i
     int64_t n_visit;       // candidates visited: positions i * stride for i < n_visit
@@ -146,43 +152,52 @@ __global__ void __launch_bounds__(1024) k_type_write(const uint8_t* __restrict__
 
 // ---------------------------------------------------------------------------
 // query vectors: q = fl32(e_h + w_r) (TransE) or fl32(e_h * w_r) (DistMult),
-// the first rounding of the screening arithmetic of every edge weight
+// the first rounding of the screening arithmetic of every edge weight.  A block
+// takes the queries q0 .. q0 + n - 1 of its chunk, each padded with zeros to dp, and
+// zero vectors up to a multiple of QP.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void load_queries(const ScanArgs& a, float* sq, float* sthr) {
+template <int QP>
+__device__ __forceinline__ int load_queries(const ScanArgs& a, int dp, float* sq, float* sthr, int* first) {
     const int d = a.g.d;
-    const int64_t total = static_cast<int64_t>(a.nq) * d;
     const bool transe = a.g.fn == MHR_SCORE_TRANSE_L1;
-    for (int64_t idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        const int qi = static_cast<int>(idx / d), j = static_cast<int>(idx - static_cast<int64_t>(qi) * d);
-        const float e = emb_f32(a.g.vemb, a.g.dtype, a.h[qi], d, j);
-        const float w = emb_f32(a.g.remb, a.g.dtype, a.r[qi], d, j);
-        sq[idx] = transe ? __fadd_rn(e, w) : __fmul_rn(e, w);
+    const int q0 = blockIdx.y * a.chunk, n = min(a.chunk, a.nq - q0);
+    for (int qi = threadIdx.x >> 5; qi < (n + QP - 1) / QP * QP; qi += kScanWarps) {
+        const bool real = qi < n;
+        const uint32_t h = real ? a.h[q0 + qi] : 0u, r = real ? a.r[q0 + qi] : 0u;
+#pragma unroll 4
+        for (int j = threadIdx.x & 31; j < dp; j += 32) {
+            float x = 0.f;
+            if (real && j < d) {
+                const float e = emb_f32(a.g.vemb, a.g.dtype, h, d, j), w = emb_f32(a.g.remb, a.g.dtype, r, d, j);
+                x = transe ? __fadd_rn(e, w) : __fmul_rn(e, w);
+            }
+            sq[static_cast<int64_t>(qi) * dp + j] = x;
+        }
     }
-    for (int qi = threadIdx.x; qi < a.nq; qi += blockDim.x) sthr[qi] = a.thr ? a.thr[qi] : -INFINITY;
+    for (int qi = threadIdx.x; qi < n + QP; qi += blockDim.x)
+        sthr[qi] = qi >= n ? INFINITY : (a.thr ? a.thr[q0 + qi] : -INFINITY);
+    if (a.thr == nullptr && blockIdx.x == 0)  // every score is kept
+        for (int qi = threadIdx.x; qi < n; qi += blockDim.x) a.cnt[q0 + qi] = static_cast<unsigned>(a.n_visit);
     __syncthreads();
-}
-
-// one survivor per qualifying lane; warp-uniform call
-__device__ __forceinline__ void append(const ScanArgs& a, int qi, bool keep, float s32, uint32_t v, int lane) {
-    const unsigned m = __ballot_sync(0xffffffffu, keep);
-    if (!m) return;
-    const int leader = __ffs(m) - 1;
-    unsigned base = 0;
-    if (lane == leader) base = atomicAdd(a.cnt + qi, static_cast<unsigned>(__popc(m)));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (keep) {
-        const unsigned pos = base + static_cast<unsigned>(__popc(m & ((1u << lane) - 1u)));
-        if (pos < static_cast<unsigned long long>(a.cap)) a.surv[static_cast<int64_t>(qi) * a.cap + pos] = SurvRec{s32, v};
-    }
+    *first = q0;
+    return n;
 }
 
 // ---------------------------------------------------------------------------
-// scan, 16-byte rows: a group of G lanes holds two adjacent candidate rows in
-// registers (lane s of the group: 16-byte vectors s, s + G, ..., NV of them per
-// row), so the group's loads of one step are G consecutive vectors of a row,
-// and every query vector load from shared memory feeds both rows.  EV elements
-// per vector (4 fp32 or 8 bf16).
+// The scans.  A lane group holds ROWS candidate rows in registers (up to 16 elements
+// of each per lane), and each query vector load from shared memory feeds all of
+// them; QP queries are scored at a time.  Their ROWS * QP partial sums are reduced
+// together: each exchange step halves the sums a lane carries, so with eight of
+// them and eight lanes every lane ends with one score and tests it.
+//
+// What bounds them: many queries, the issue of the fp32 pipe (TransE: half a paired
+// subtraction and an addition per element); a few, the rows' bandwidth.  64 queries
+// x 167,000 candidates of 128 fp32 values, TransE: 247 us (two rows, each sum reduced
+// and tested by itself) -> 131 us, the sample's 8,192 candidates 55 -> 15 us by
+// cutting the queries into chunks as well; one query over 1M candidates 75 us, 6.8
+// TB/s, before and after.
 // ---------------------------------------------------------------------------
+
 template <bool BF16>
 __device__ __forceinline__ void unpack_row(const uint4& w, float* x) {
     if constexpr (BF16) {
@@ -202,112 +217,223 @@ __device__ __forceinline__ void unpack_row(const uint4& w, float* x) {
     }
 }
 
-template <bool TRANSE>
-__device__ __forceinline__ float term32(float q, float c) {
-    if constexpr (TRANSE) return fabsf(__fsub_rn(q, c));
-    else return q * c;
+// The score of query qi for candidate i of the visit order, on the lanes with
+// `mine`.  Keep-every-score mode (no threshold): candidate i owns slot i, no counter
+// needed; otherwise the few lanes that pass append, one counter update per query.
+__device__ __forceinline__ void emit(const ScanArgs& a, int qi, bool mine, float s32, int64_t i, int lane, float thr) {
+    const bool keep = mine && s32 >= thr;
+    const unsigned m = __ballot_sync(0xffffffffu, keep);
+    if (!keep) return;
+    const int64_t at = i * a.stride;
+    const uint32_t v = a.cand ? __ldg(a.cand + at) : static_cast<uint32_t>(at);
+    int64_t pos = i;
+    if (a.thr) {
+        const unsigned peers = __match_any_sync(m, qi);
+        const int leader = __ffs(peers) - 1;
+        unsigned base = 0;
+        if (lane == leader) base = atomicAdd(a.cnt + qi, static_cast<unsigned>(__popc(peers)));
+        pos = __shfl_sync(peers, base, leader) + static_cast<unsigned>(__popc(peers & ((1u << lane) - 1u)));
+        if (pos >= a.cap) return;
+    }
+    a.surv[static_cast<int64_t>(qi) * a.cap + pos] = SurvRec{s32, v};
 }
 
-// keep-every-score mode (no threshold): candidate i of the visit order owns
-// slot i, no counter needed; otherwise a warp-aggregated append
-__device__ __forceinline__ void emit(const ScanArgs& a, int qi, bool valid, bool leader, float s32, uint32_t v,
-                                     int64_t i, int lane, float thr) {
-    if (a.thr == nullptr) {
-        if (valid && leader) a.surv[static_cast<int64_t>(qi) * a.cap + i] = SurvRec{s32, v};
+// two fp32 operations at once (a 64-bit register pair), each rounded as by itself
+__device__ __forceinline__ float2 sub2(float2 x, float2 y) {
+    float2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long&>(r))
+        : "l"(reinterpret_cast<unsigned long long&>(x)), "l"(reinterpret_cast<unsigned long long&>(y)));
+    return r;
+}
+__device__ __forceinline__ float2 fma2(float2 x, float2 y, float2 z) {
+    float2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long&>(r))
+        : "l"(reinterpret_cast<unsigned long long&>(x)), "l"(reinterpret_cast<unsigned long long&>(y)),
+          "l"(reinterpret_cast<unsigned long long&>(z)));
+    return r;
+}
+
+// acc[r] += the row's terms of two elements: TransE into acc[r].x, DistMult into both halves
+template <bool TRANSE>
+__device__ __forceinline__ void add_terms(float2& acc, float2 q, float2 x) {
+    if constexpr (TRANSE) {
+        const float2 t = sub2(q, x);
+        acc.x += fabsf(t.x);
+        acc.y += fabsf(t.y);
     } else {
-        append(a, qi, valid && leader && s32 >= thr, s32, v, lane);
+        acc = fma2(q, x, acc);
     }
 }
 
-__device__ __forceinline__ void keep_all_counts(const ScanArgs& a) {
-    if (a.thr == nullptr && blockIdx.x == 0)
-        for (int qi = threadIdx.x; qi < a.nq; qi += blockDim.x) a.cnt[qi] = static_cast<unsigned>(a.n_visit);
+// Sums over a group of G lanes of N values per lane.  L exchange steps (2^L <= G, N)
+// leave N >> L sums per lane: value (returned index + j) in v[j], each on the lanes
+// s < 2^L and their repetitions.
+template <int N, int L>
+__device__ __forceinline__ int reduce_group(float (&v)[N], int s, int G) {
+    int first = 0;
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+        const int half = N >> (k + 1);
+        const bool hi = ((s >> k) & 1) != 0;
+#pragma unroll
+        for (int j = 0; j < half; ++j) {
+            const float send = hi ? v[j] : v[j + half], keep = hi ? v[j + half] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, send, 1 << k);
+        }
+        first += hi ? half : 0;
+    }
+    for (int o = 1 << L; o < G; o <<= 1) {
+#pragma unroll
+        for (int j = 0; j < (N >> L); ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+    }
+    return first;
 }
 
-template <int NV, bool BF16, bool TRANSE>
-__global__ void __launch_bounds__(kScanThreads) k_tail_scan(ScanArgs a) {
+// the scores of ROWS rows from i0 for QP queries from qi (values q * ROWS + row)
+template <int ROWS, int QP, int L, bool TRANSE>
+__device__ __forceinline__ void finish_rows(const ScanArgs& a, float (&v)[ROWS * QP], int s, int G, int64_t i0, int q0,
+                                            int qi, const float* sthr, int lane) {
+    const int first = reduce_group<ROWS * QP, L>(v, s, G);
+#pragma unroll
+    for (int j = 0; j < ((ROWS * QP) >> L); ++j) {
+        const int id = first + j, q = qi + id / ROWS;
+        const int64_t i = i0 + id % ROWS;
+        emit(a, q0 + q, s < (1 << L) && i < a.n_visit, TRANSE ? __fsub_rn(a.g.gamma32, v[j]) : v[j], i, lane, sthr[q]);
+    }
+}
+
+// rows of whole 16-byte vectors: lane s of a group holds vectors s, s + G, ... (NV of
+// them per row), so the group's loads of one step are consecutive.  Rows and query
+// vectors are padded with zeros to G * NV vectors, whose terms are zero.  G >= 2^L.
+template <int NV, int ROWS, int QP, int L, bool BF16, bool TRANSE>
+__global__ void __launch_bounds__(kScanThreads, ROWS == 2 ? 4 : 2) k_tail_scan(const __grid_constant__ ScanArgs a) {
     extern __shared__ float4 smem4[];
     float* sq = reinterpret_cast<float*>(smem4);
-    const int d = a.g.d, nq = a.nq;
-    float* sthr = sq + static_cast<int64_t>(nq) * d;
-    load_queries(a, sq, sthr);
-    keep_all_counts(a);
-
     constexpr int EV = BF16 ? 8 : 4;
+    const int d = a.g.d, G = a.G, dp = G * NV * EV;
+    float* sthr = sq + static_cast<int64_t>((a.chunk + QP - 1) / QP * QP) * dp;
+    int q0;
+    const int nq = load_queries<QP>(a, dp, sq, sthr, &q0);
+
     const int dv = d / EV;
-    const int G = a.G;
     const int lane = threadIdx.x & 31;
     const int s = lane & (G - 1);
     const int grp = lane / G;
-    const int cpw = 2 * (32 / G);
+    const int cpw = ROWS * (32 / G);
     const int64_t ntiles = (a.n_visit + cpw - 1) / cpw;
     const int64_t nwarps = static_cast<int64_t>(gridDim.x) * kScanWarps;
     const size_t row_bytes = static_cast<size_t>(d) * (BF16 ? 2 : 4);
-    const float gamma32 = a.g.gamma32;
 
     for (int64_t t = static_cast<int64_t>(blockIdx.x) * kScanWarps + (threadIdx.x >> 5); t < ntiles; t += nwarps) {
-        const int64_t i0 = t * cpw + 2 * grp, i1 = i0 + 1;
-        const bool valid0 = i0 < a.n_visit, valid1 = i1 < a.n_visit;
-        uint32_t v0 = 0, v1 = 0;
-        if (valid0) v0 = a.cand ? __ldg(a.cand + i0 * a.stride) : static_cast<uint32_t>(i0 * a.stride);
-        if (valid1) v1 = a.cand ? __ldg(a.cand + i1 * a.stride) : static_cast<uint32_t>(i1 * a.stride);
-        const uint4* row0 = reinterpret_cast<const uint4*>(static_cast<const char*>(a.g.vemb) + v0 * row_bytes);
-        const uint4* row1 = reinterpret_cast<const uint4*>(static_cast<const char*>(a.g.vemb) + v1 * row_bytes);
-        float x0[NV * EV], x1[NV * EV];
+        const int64_t i0 = t * cpw + ROWS * grp;
+        float x[ROWS][NV * EV];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            const int vi = s + G * k;
-            uint4 w0 = make_uint4(0u, 0u, 0u, 0u), w1 = w0;
-            if (valid0 && vi < dv) w0 = __ldg(row0 + vi);
-            if (valid1 && vi < dv) w1 = __ldg(row1 + vi);
-            unpack_row<BF16>(w0, x0 + k * EV);
-            unpack_row<BF16>(w1, x1 + k * EV);
-        }
-        for (int qi = 0; qi < nq; ++qi) {
-            const float4* q4 = reinterpret_cast<const float4*>(sq + static_cast<int64_t>(qi) * d);
-            float acc0 = 0.f, acc1 = 0.f;
+        for (int r = 0; r < ROWS; ++r) {
+            const int64_t i = i0 + r;
+            const bool valid = i < a.n_visit;
+            uint32_t v = 0;
+            if (valid) v = a.cand ? __ldg(a.cand + i * a.stride) : static_cast<uint32_t>(i * a.stride);
+            const uint4* row = reinterpret_cast<const uint4*>(static_cast<const char*>(a.g.vemb) + v * row_bytes);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
                 const int vi = s + G * k;
-                if (vi < dv) {
+                unpack_row<BF16>(valid && vi < dv ? __ldg(row + vi) : make_uint4(0u, 0u, 0u, 0u), x[r] + k * EV);
+            }
+        }
+        const float4* q4 = reinterpret_cast<const float4*>(sq) + s * (EV / 4);
+        for (int qi = 0; qi < nq; qi += QP, q4 += QP * (dp / 4)) {
+            float2 acc[QP][ROWS];
 #pragma unroll
-                    for (int e4 = 0; e4 < EV / 4; ++e4) {
-                        const float4 qq = q4[vi * (EV / 4) + e4];
-                        const float* y0 = x0 + k * EV + e4 * 4;
-                        const float* y1 = x1 + k * EV + e4 * 4;
-                        acc0 += term32<TRANSE>(qq.x, y0[0]);
-                        acc1 += term32<TRANSE>(qq.x, y1[0]);
-                        acc0 += term32<TRANSE>(qq.y, y0[1]);
-                        acc1 += term32<TRANSE>(qq.y, y1[1]);
-                        acc0 += term32<TRANSE>(qq.z, y0[2]);
-                        acc1 += term32<TRANSE>(qq.z, y1[2]);
-                        acc0 += term32<TRANSE>(qq.w, y0[3]);
-                        acc1 += term32<TRANSE>(qq.w, y1[3]);
+            for (int q = 0; q < QP; ++q)
+#pragma unroll
+                for (int r = 0; r < ROWS; ++r) acc[q][r] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < NV; ++k)
+#pragma unroll
+                for (int e4 = 0; e4 < EV / 4; ++e4)
+#pragma unroll
+                    for (int q = 0; q < QP; ++q) {
+                        const float4 qq = q4[q * (dp / 4) + G * k * (EV / 4) + e4];
+#pragma unroll
+                        for (int r = 0; r < ROWS; ++r) {
+                            const float* y = x[r] + k * EV + e4 * 4;
+                            add_terms<TRANSE>(acc[q][r], make_float2(qq.x, qq.y), make_float2(y[0], y[1]));
+                            add_terms<TRANSE>(acc[q][r], make_float2(qq.z, qq.w), make_float2(y[2], y[3]));
+                        }
                     }
-                }
-            }
-            for (int o = G >> 1; o > 0; o >>= 1) {
-                acc0 += __shfl_xor_sync(0xffffffffu, acc0, o);
-                acc1 += __shfl_xor_sync(0xffffffffu, acc1, o);
-            }
-            const float s0 = TRANSE ? __fsub_rn(gamma32, acc0) : acc0;
-            const float s1 = TRANSE ? __fsub_rn(gamma32, acc1) : acc1;
-            const float thr = sthr[qi];
-            emit(a, qi, valid0, s == 0, s0, v0, i0, lane, thr);
-            emit(a, qi, valid1, s == 0, s1, v1, i1, lane, thr);
+            float v[ROWS * QP];
+#pragma unroll
+            for (int q = 0; q < QP; ++q)
+#pragma unroll
+                for (int r = 0; r < ROWS; ++r) v[q * ROWS + r] = acc[q][r].x + acc[q][r].y;
+            finish_rows<ROWS, QP, L, TRANSE>(a, v, s, G, i0, q0, qi, sthr, lane);
         }
     }
 }
 
-// scan, any row length: one warp per candidate, lanes stride over the row
-template <bool TRANSE>
-__global__ void __launch_bounds__(kScanThreads) k_tail_scan_any(ScanArgs a) {
+// rows of up to 32 * KX elements of any length: a warp per ROWS rows, lane s holds
+// elements s, s + 32, ...
+template <int KX, int ROWS, int QP, bool TRANSE>
+__global__ void __launch_bounds__(kScanThreads, 2) k_tail_scan_el(const __grid_constant__ ScanArgs a) {
     extern __shared__ float4 smem4[];
     float* sq = reinterpret_cast<float*>(smem4);
-    const int d = a.g.d, nq = a.nq;
-    float* sthr = sq + static_cast<int64_t>(nq) * d;
-    load_queries(a, sq, sthr);
-    keep_all_counts(a);
+    const int d = a.g.d;
+    constexpr int dp = 32 * KX, L = ROWS * QP == 8 ? 3 : 1;
+    static_assert(ROWS * QP == 8 || ROWS * QP == 2, "exchange steps for eight sums or two");
+    float* sthr = sq + static_cast<int64_t>((a.chunk + QP - 1) / QP * QP) * dp;
+    int q0;
+    const int nq = load_queries<QP>(a, dp, sq, sthr, &q0);
+    const int lane = threadIdx.x & 31;
+    const int64_t ntiles = (a.n_visit + ROWS - 1) / ROWS;
+    const int64_t nwarps = static_cast<int64_t>(gridDim.x) * kScanWarps;
+    for (int64_t t = static_cast<int64_t>(blockIdx.x) * kScanWarps + (threadIdx.x >> 5); t < ntiles; t += nwarps) {
+        const int64_t i0 = t * ROWS;
+        float x[ROWS][KX];
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const int64_t i = i0 + r;
+            const bool valid = i < a.n_visit;
+            uint32_t v = 0;
+            if (valid) v = a.cand ? __ldg(a.cand + i * a.stride) : static_cast<uint32_t>(i * a.stride);
+#pragma unroll
+            for (int k = 0; k < KX; ++k) {
+                const int j = lane + 32 * k;
+                x[r][k] = valid && j < d ? emb_f32(a.g.vemb, a.g.dtype, v, d, j) : 0.f;
+            }
+        }
+        const float* sv = sq + lane;
+        for (int qi = 0; qi < nq; qi += QP, sv += QP * dp) {
+            float v[ROWS * QP];
+#pragma unroll
+            for (int j = 0; j < ROWS * QP; ++j) v[j] = 0.f;
+#pragma unroll
+            for (int k = 0; k < KX; ++k)
+#pragma unroll
+                for (int q = 0; q < QP; ++q) {
+                    const float qq = sv[q * dp + 32 * k];
+#pragma unroll
+                    for (int r = 0; r < ROWS; ++r) {
+                        float& c = v[q * ROWS + r];
+                        if constexpr (TRANSE) c += fabsf(__fsub_rn(qq, x[r][k]));
+                        else c += qq * x[r][k];
+                    }
+                }
+            finish_rows<ROWS, QP, L, TRANSE>(a, v, lane, 32, i0, q0, qi, sthr, lane);
+        }
+    }
+}
+
+// longer rows: one warp per candidate, the row read again for each query
+template <bool TRANSE>
+__global__ void __launch_bounds__(kScanThreads) k_tail_scan_any(const __grid_constant__ ScanArgs a) {
+    extern __shared__ float4 smem4[];
+    float* sq = reinterpret_cast<float*>(smem4);
+    const int d = a.g.d;
+    float* sthr = sq + static_cast<int64_t>(a.chunk) * d;
+    int q0;
+    const int nq = load_queries<1>(a, d, sq, sthr, &q0);
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = static_cast<int64_t>(gridDim.x) * kScanWarps;
     const float gamma32 = a.g.gamma32;
@@ -323,8 +449,7 @@ __global__ void __launch_bounds__(kScanThreads) k_tail_scan_any(ScanArgs a) {
                 else acc += q[j] * c;
             }
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            const float s32 = TRANSE ? __fsub_rn(gamma32, acc) : acc;
-            emit(a, qi, true, lane == 0, s32, v, i, lane, sthr[qi]);
+            emit(a, q0 + qi, lane == 0, TRANSE ? __fsub_rn(gamma32, acc) : acc, i, lane, sthr[qi]);
         }
     }
 }
@@ -463,7 +588,7 @@ __device__ __forceinline__ bool ranks_before(const BandRec& x, const BandRec& y)
 constexpr int kQ64Max = 2048;  // rows up to this length use the shared fp64 query vector
 
 template <bool TRANSE>
-__device__ __forceinline__ double term64(double q, float c) {
+__device__ __forceinline__ double row_term64(double q, float c) {
     if constexpr (TRANSE) return fabs(__dsub_rn(q, static_cast<double>(c)));
     else return __dmul_rn(q, static_cast<double>(c));
 }
@@ -481,10 +606,10 @@ __device__ double rescore_row(const DevGraph& g, const double* q64, uint32_t v) 
         for (int j4 = 0; j4 < (d >> 2); ++j4) {
             const float4 c = __ldg(c4 + j4);
             const double* q = q64 + 4 * j4;
-            acc = __dadd_rn(acc, term64<TRANSE>(q[0], c.x));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[1], c.y));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[2], c.z));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[3], c.w));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[0], c.x));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[1], c.y));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[2], c.z));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[3], c.w));
         }
     } else if (g.dtype == MHR_BF16 && (d & 7) == 0) {
         const uint4* c8 = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(g.vemb) + static_cast<int64_t>(v) * d);
@@ -492,17 +617,17 @@ __device__ double rescore_row(const DevGraph& g, const double* q64, uint32_t v) 
         for (int j8 = 0; j8 < (d >> 3); ++j8) {
             const uint4 w = __ldg(c8 + j8);
             const double* q = q64 + 8 * j8;
-            acc = __dadd_rn(acc, term64<TRANSE>(q[0], bf_lo(w.x)));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[1], bf_hi(w.x)));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[2], bf_lo(w.y)));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[3], bf_hi(w.y)));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[4], bf_lo(w.z)));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[5], bf_hi(w.z)));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[6], bf_lo(w.w)));
-            acc = __dadd_rn(acc, term64<TRANSE>(q[7], bf_hi(w.w)));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[0], bf_lo(w.x)));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[1], bf_hi(w.x)));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[2], bf_lo(w.y)));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[3], bf_hi(w.y)));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[4], bf_lo(w.z)));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[5], bf_hi(w.z)));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[6], bf_lo(w.w)));
+            acc = __dadd_rn(acc, row_term64<TRANSE>(q[7], bf_hi(w.w)));
         }
     } else {
-        for (int j = 0; j < d; ++j) acc = __dadd_rn(acc, term64<TRANSE>(q64[j], emb_f32(g.vemb, g.dtype, v, d, j)));
+        for (int j = 0; j < d; ++j) acc = __dadd_rn(acc, row_term64<TRANSE>(q64[j], emb_f32(g.vemb, g.dtype, v, d, j)));
     }
     return TRANSE ? __dsub_rn(g.gamma, acc) : acc;
 }
@@ -513,7 +638,7 @@ __global__ void __launch_bounds__(kFinalThreads)
                  BandRec* __restrict__ band, int K, double E2, mhr_tail* __restrict__ out,
                  int32_t* __restrict__ n_out, unsigned* __restrict__ band_cnt) {
     __shared__ SelectSmem sm;
-    extern __shared__ BandRec sbuf[];  // kSortMax records, then the fp64 query vector
+    extern __shared__ __align__(16) BandRec sbuf[];  // kSortMax records, then the fp64 query vector
     double* q64 = reinterpret_cast<double*>(sbuf + kSortMax);
     const int q = blockIdx.x;
     if (static_cast<int64_t>(cnt[q]) > cap) return;  // overflowed: rescanned alone by the host
@@ -545,16 +670,61 @@ __global__ void __launch_bounds__(kFinalThreads)
     }
     __syncthreads();
     const unsigned nb = sm.count;
-    // fp64 rescoring, one band member per thread over dense warps
-    for (unsigned p = threadIdx.x; p < nb; p += blockDim.x) {
-        const uint32_t v = b[p].v;
-        double w;
-        if (!shared_q) w = edge_w64(g, hq, rq, v);
-        else if (transe) w = rescore_row<true>(g, q64, v);
-        else w = rescore_row<false>(g, q64, v);
-        b[p] = BandRec{w, v, 0u};
+    // fp64 rescoring: TransE a warp per member, in integers; members the integers do
+    // not hold, and DistMult, one per thread over dense warps
+    __syncthreads();  // everyone has nb
+    if (threadIdx.x == 0) sm.count = 0u;
+    __syncthreads();
+    if (transe) {
+        const int lane = threadIdx.x & 31;
+#pragma unroll 2
+        for (unsigned p = threadIdx.x >> 5; p < nb; p += kFinalThreads / 32) {
+            const uint32_t v = b[p].v;
+            bool ok;
+            const double w = warp_w64_fixed(g, hq, rq, v, lane, &ok);
+            if (lane == 0) {
+                b[p] = BandRec{w, v, ok ? 0u : 1u};
+                if (!ok) sm.count = 1u;
+            }
+        }
+        __syncthreads();
+    }
+    if (!transe || sm.count) {
+        for (unsigned p = threadIdx.x; p < nb; p += blockDim.x) {
+            const uint32_t v = b[p].v;
+            if (transe && b[p].pad == 0u) continue;
+            double w;
+            if (!shared_q) w = edge_w64(g, hq, rq, v);
+            else if (transe) w = rescore_row<true>(g, q64, v);
+            else w = rescore_row<false>(g, q64, v);
+            b[p] = BandRec{w, v, 0u};
+        }
     }
     __syncthreads();
+
+    // a short band: a record's place is the number of records before it
+    if (nb <= static_cast<unsigned>(kRankMax)) {
+        uint64_t* keys = reinterpret_cast<uint64_t*>(sbuf);  // (score key, vertex), two words a record
+        for (unsigned i = threadIdx.x; i < nb; i += blockDim.x) {
+            keys[2 * i] = score_key(b[i].w);
+            keys[2 * i + 1] = b[i].v;
+        }
+        __syncthreads();
+        for (unsigned i = threadIdx.x; i < nb; i += blockDim.x) {
+            const uint64_t hi = keys[2 * i], v = keys[2 * i + 1];
+            int rank = 0;
+            for (unsigned j = 0; j < nb; ++j) {
+                const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(keys + 2 * j);
+                rank += o.x > hi || (o.x == hi && o.y < v) ? 1 : 0;
+            }
+            if (rank < K) out[static_cast<int64_t>(q) * K + rank] = mhr_tail{b[i].w, static_cast<uint32_t>(v), 0u};
+        }
+        if (threadIdx.x == 0) {
+            n_out[q] = static_cast<int32_t>(min(nb, static_cast<unsigned>(K)));
+            band_cnt[q] = nb;
+        }
+        return;
+    }
 
     // 2. the records to sort: the whole band, or exactly its K best
     unsigned m;
@@ -636,64 +806,123 @@ cudaError_t grow(void** p, size_t* have, size_t want) {
 struct ScanKernel {
     void (*fn)(ScanArgs) = nullptr;
     int G = 1;
-    int rows_per_group = 1;
+    int dp = 0;    // floats of a query vector in shared memory
+    int qp = 1;    // queries scored at a time
+    int rows = 1;  // candidates a warp takes at a time
+    int per_sm = 1;
 };
 
-ScanKernel pick_scan(const DevGraph& dg) {
-    const bool transe = dg.fn == MHR_SCORE_TRANSE_L1;
-    const int d = dg.d;
-    const bool bf = dg.dtype == MHR_BF16;
-    // two rows per lane group: at most 16 elements of each row per lane
-    const int ev = bf ? 8 : 4, nvmax = bf ? 2 : 4;
+template <int NV, int ROWS, int QP, int L, bool BF16>
+void use_scan(ScanKernel& k, bool transe, int G) {
+    k.fn = transe ? k_tail_scan<NV, ROWS, QP, L, BF16, true> : k_tail_scan<NV, ROWS, QP, L, BF16, false>;
+    k.G = G;
+    k.dp = G * NV * (BF16 ? 8 : 4);
+    k.qp = QP;
+    k.rows = ROWS * (32 / G);
+}
+
+template <int ROWS, int QP>
+void use_scan_vec(ScanKernel& k, const DevGraph& dg) {
+    constexpr int N = ROWS * QP, L = N == 8 ? 3 : 1;
+    const bool transe = dg.fn == MHR_SCORE_TRANSE_L1, bf = dg.dtype == MHR_BF16;
+    const int dv = dg.d / (bf ? 8 : 4), nvmax = bf ? 2 : 4;
+    int G = 1;
+    while ((dv + G - 1) / G > nvmax) G <<= 1;
+    if (G == 1) {
+        if (bf) use_scan<2, ROWS, QP, 0, true>(k, transe, G);
+        else use_scan<4, ROWS, QP, 0, false>(k, transe, G);
+    } else if (G == 2 || L == 1) {
+        if (bf) use_scan<2, ROWS, QP, 1, true>(k, transe, G);
+        else use_scan<4, ROWS, QP, 1, false>(k, transe, G);
+    } else if (G == 4) {
+        if (bf) use_scan<2, ROWS, QP, L == 3 ? 2 : L, true>(k, transe, G);
+        else use_scan<4, ROWS, QP, L == 3 ? 2 : L, false>(k, transe, G);
+    } else {
+        if (bf) use_scan<2, ROWS, QP, L, true>(k, transe, G);
+        else use_scan<4, ROWS, QP, L, false>(k, transe, G);
+    }
+}
+
+template <int KX>
+void use_scan_el(ScanKernel& k, bool transe, bool few) {
+    if (few) k.fn = transe ? k_tail_scan_el<KX, 2, 1, true> : k_tail_scan_el<KX, 2, 1, false>;
+    else k.fn = transe ? k_tail_scan_el<KX, 4, 2, true> : k_tail_scan_el<KX, 4, 2, false>;
+    k.G = 32;
+    k.dp = 32 * KX;
+    k.qp = few ? 1 : 2;
+    k.rows = few ? 2 : 4;
+}
+
+// Whole vectors where the rows have them: as few lanes per row as hold it in 16
+// elements each.  Otherwise element by element, up to 16 per lane.  Up to four
+// queries the rows' bandwidth bounds the scan, and two rows per group with more
+// warps in flight read them faster (one query over 1M rows of 512 bytes: 77 us, four
+// rows 89 us); beyond, eight sums at a time take a third fewer instructions.
+ScanKernel pick_scan(const DevGraph& dg, int nq) {
+    const bool transe = dg.fn == MHR_SCORE_TRANSE_L1, bf = dg.dtype == MHR_BF16;
+    const int d = dg.d, ev = bf ? 8 : 4, nvmax = bf ? 2 : 4;
+    const bool few = nq <= 4;
     ScanKernel k;
     if (d % ev == 0 && d / ev <= 32 * nvmax) {
-        const int dv = d / ev;
-        int G = 1;
-        while ((dv + G - 1) / G > nvmax) G <<= 1;
-        const int need = (dv + G - 1) / G;
-        int NV = 1;
-        while (NV < need) NV <<= 1;
-        k.G = G;
-        k.rows_per_group = 2;
-        if (bf) {
-            if (NV == 1) k.fn = transe ? k_tail_scan<1, true, true> : k_tail_scan<1, true, false>;
-            else k.fn = transe ? k_tail_scan<2, true, true> : k_tail_scan<2, true, false>;
-        } else {
-            if (NV == 1) k.fn = transe ? k_tail_scan<1, false, true> : k_tail_scan<1, false, false>;
-            else if (NV == 2) k.fn = transe ? k_tail_scan<2, false, true> : k_tail_scan<2, false, false>;
-            else k.fn = transe ? k_tail_scan<4, false, true> : k_tail_scan<4, false, false>;
-        }
+        if (few) use_scan_vec<2, 1>(k, dg);
+        else use_scan_vec<4, 2>(k, dg);
         return k;
     }
-    k.G = 32;
-    k.rows_per_group = 1;
-    k.fn = transe ? k_tail_scan_any<true> : k_tail_scan_any<false>;
+    if (d <= 32) use_scan_el<1>(k, transe, few);
+    else if (d <= 64) use_scan_el<2>(k, transe, few);
+    else if (d <= 128) use_scan_el<4>(k, transe, few);
+    else if (d <= 256) use_scan_el<8>(k, transe, few);
+    else if (d <= 512) use_scan_el<16>(k, transe, few);
+    else {
+        k.fn = transe ? k_tail_scan_any<true> : k_tail_scan_any<false>;
+        k.G = 32;
+        k.dp = d;
+    }
     return k;
+}
+
+// shared memory of a block that takes n queries
+size_t scan_smem(const ScanKernel& sk, int n) {
+    const size_t whole = (n + sk.qp - 1) / sk.qp * sk.qp;
+    return whole * sk.dp * 4 + (whole + sk.qp) * 4;
+}
+
+// most queries a block takes: their vectors fit the query buffer (one iteration's always do)
+int scan_fit(const ScanKernel& sk) {
+    const size_t n = kQueryBytes / (static_cast<size_t>(sk.dp) * 4 + 4);
+    return static_cast<int>(std::max<size_t>(sk.qp, n / sk.qp * sk.qp));
 }
 
 // Host-side set-up of the scan kernel for launches of up to nq_max queries:
 // the shared-memory attribute and the resident blocks per SM.  Done once per
 // call, before any event is recorded, so event times cover device work only.
-mhr_status scan_setup(const mhr_graph* g, const ScanKernel& sk, int nq_max, int* per_sm) {
-    const size_t smem = static_cast<size_t>(nq_max) * g->dg.d * 4 + static_cast<size_t>(nq_max) * 4;
+mhr_status scan_setup(ScanKernel& sk, int nq_max) {
+    const size_t smem = scan_smem(sk, std::min(nq_max, scan_fit(sk)));
     MHR_CUDA_TRY(cudaFuncSetAttribute(sk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
     int n = 0;
     MHR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sk.fn, kScanThreads, smem));
-    *per_sm = std::max(1, n);
+    sk.per_sm = std::max(1, n);
     return MHR_OK;
 }
 
-// a.nq <= the nq_max given to scan_setup, whose per_sm this takes
-mhr_status launch_scan(const mhr_graph* g, const ScanKernel& sk, const ScanArgs& a, int per_sm, cudaStream_t st) {
+// a.nq <= the nq_max given to scan_setup.  The queries are cut into chunks until
+// every resident warp has about eight units of a tile and a chunk (an uneven last
+// one then costs a tenth at most), down to eight queries, whose arithmetic still
+// covers loading the tile's rows once more per chunk.
+mhr_status launch_scan(const mhr_graph* g, const ScanKernel& sk, const ScanArgs& a, cudaStream_t st) {
     if (a.nq <= 0 || a.n_visit <= 0) return MHR_OK;
-    const size_t smem = static_cast<size_t>(a.nq) * g->dg.d * 4 + static_cast<size_t>(a.nq) * 4;
-    const int cpw = sk.rows_per_group * (32 / sk.G);
-    const int64_t ntiles = (a.n_visit + cpw - 1) / cpw;
-    const int64_t need = (ntiles + kScanWarps - 1) / kScanWarps;
-    const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(need, int64_t(std::max(1, g->num_sms)) * per_sm)));
+    const int64_t ntiles = (a.n_visit + sk.rows - 1) / sk.rows;
+    const int64_t blocks = int64_t(std::max(1, g->num_sms)) * sk.per_sm;
+    int64_t chunks = std::min<int64_t>((8 * blocks * kScanWarps + ntiles - 1) / ntiles, (a.nq + 7) / 8);
+    chunks = std::max<int64_t>({int64_t(1), chunks, (a.nq + scan_fit(sk) - 1) / scan_fit(sk)});
     ScanArgs b = a;
     b.G = sk.G;
-    sk.fn<<<grid, kScanThreads, smem, st>>>(b);
+    b.chunk = static_cast<int>((a.nq + chunks - 1) / chunks + sk.qp - 1) / sk.qp * sk.qp;
+    chunks = (a.nq + b.chunk - 1) / b.chunk;
+    const int64_t need = (ntiles + kScanWarps - 1) / kScanWarps;
+    const dim3 grid(static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(need, blocks / chunks))),
+                    static_cast<unsigned>(chunks));
+    sk.fn<<<grid, kScanThreads, scan_smem(sk, b.chunk), st>>>(b);
     MHR_CUDA_TRY(cudaGetLastError());
     return MHR_OK;
 }
@@ -754,26 +983,37 @@ extern "C" mhr_status mhr_tail_topk(const mhr_graph* gc, int32_t nq, const uint3
     if (!h || !r || !out || !n_out) return fail(MHR_EINVAL, "NULL array");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
 
+    if (!g->tail) g->tail = new TailCache();
+    TailCache* tc = g->tail;
+    if (!tc->pinned) MHR_CUDA_TRY(cudaMallocHost(reinterpret_cast<void**>(&tc->pinned), kPinned));
+    if (stats)
+        for (cudaEvent_t& e : tc->ev)
+            if (!e) MHR_CUDA_TRY(cudaEventCreate(&e));
+
     // validate the queries on the host (a short copy when they live on the device)
-    std::vector<uint32_t> hh(nq);
-    std::vector<uint16_t> hr(nq);
-    if (mem == MHR_MEM_HOST) {
-        std::copy(h, h + nq, hh.begin());
-        std::copy(r, r + nq, hr.begin());
-    } else {
-        MHR_CUDA_TRY(cudaMemcpyAsync(hh.data(), h, 4ull * nq, cudaMemcpyDeviceToHost, st));
-        MHR_CUDA_TRY(cudaMemcpyAsync(hr.data(), r, 2ull * nq, cudaMemcpyDeviceToHost, st));
+    std::vector<uint32_t> vh;
+    std::vector<uint16_t> vr;
+    const uint32_t* hh = h;
+    const uint16_t* hr = r;
+    if (mem == MHR_MEM_DEVICE) {
+        uint32_t* ph = reinterpret_cast<uint32_t*>(tc->pinned);
+        uint16_t* pr = reinterpret_cast<uint16_t*>(ph + nq);
+        if (6ull * nq > kPinned) {
+            vh.resize(nq);
+            vr.resize(nq);
+            ph = vh.data();
+            pr = vr.data();
+        }
+        MHR_CUDA_TRY(cudaMemcpyAsync(ph, h, 4ull * nq, cudaMemcpyDeviceToHost, st));
+        MHR_CUDA_TRY(cudaMemcpyAsync(pr, r, 2ull * nq, cudaMemcpyDeviceToHost, st));
         MHR_CUDA_TRY(cudaStreamSynchronize(st));
+        hh = ph;
+        hr = pr;
     }
     for (int i = 0; i < nq; ++i) {
         if (static_cast<int64_t>(hh[i]) >= g->dg.n) return fail(MHR_EINVAL, "head out of range");
         if (static_cast<int32_t>(hr[i]) >= g->dg.R) return fail(MHR_EINVAL, "relation out of range");
     }
-
-    if (!g->tail) g->tail = new TailCache();
-    TailCache* tc = g->tail;
-    for (cudaEvent_t& e : tc->ev)
-        if (!e) MHR_CUDA_TRY(cudaEventCreate(&e));
 
     const uint32_t* cand = nullptr;
     int64_t Nc = g->dg.n;
@@ -803,8 +1043,8 @@ extern "C" mhr_status mhr_tail_topk(const mhr_graph* gc, int32_t nq, const uint3
         return o;
     };
     const size_t o_h = carve(4ull * nq), o_r = carve(2ull * nq), o_out = carve(sizeof(mhr_tail) * nq * K),
-                 o_nout = carve(4ull * nq), o_thr = carve(4ull * QB), o_cnt = carve(4ull * QB * 2),
-                 o_bc = carve(4ull * QB), o_sa = carve(sizeof(SurvRec) * QB * capA),
+                 o_nout = carve(4ull * nq), o_thr = carve(4ull * QB), o_cnt = carve(4ull * QB * 3),
+                 o_sa = carve(sizeof(SurvRec) * QB * capA),
                  o_sb = carve(sizeof(SurvRec) * QB * capB), o_band = carve(sizeof(BandRec) * QB * capB);
     MHR_CUDA_TRY(grow(&tc->scratch, &tc->scratch_bytes, off));
     char* base = static_cast<char*>(tc->scratch);
@@ -813,14 +1053,14 @@ extern "C" mhr_status mhr_tail_topk(const mhr_graph* gc, int32_t nq, const uint3
     mhr_tail* d_out = reinterpret_cast<mhr_tail*>(base + o_out);
     int32_t* d_nout = reinterpret_cast<int32_t*>(base + o_nout);
     float* d_thr = reinterpret_cast<float*>(base + o_thr);
-    unsigned* d_cnt = reinterpret_cast<unsigned*>(base + o_cnt);  // [QB] sample, [QB] full pass
-    unsigned* d_bc = reinterpret_cast<unsigned*>(base + o_bc);
+    unsigned* d_cnt = reinterpret_cast<unsigned*>(base + o_cnt);  // [QB] sample, [QB] full pass, [QB] band
+    unsigned* d_bc = d_cnt + 2 * QB;
     SurvRec* d_sa = reinterpret_cast<SurvRec*>(base + o_sa);
     SurvRec* d_sb = reinterpret_cast<SurvRec*>(base + o_sb);
     BandRec* d_band = reinterpret_cast<BandRec*>(base + o_band);
     if (mem == MHR_MEM_HOST) {
-        MHR_CUDA_TRY(cudaMemcpyAsync(d_h, hh.data(), 4ull * nq, cudaMemcpyHostToDevice, st));
-        MHR_CUDA_TRY(cudaMemcpyAsync(d_r, hr.data(), 2ull * nq, cudaMemcpyHostToDevice, st));
+        MHR_CUDA_TRY(cudaMemcpyAsync(d_h, h, 4ull * nq, cudaMemcpyHostToDevice, st));
+        MHR_CUDA_TRY(cudaMemcpyAsync(d_r, r, 2ull * nq, cudaMemcpyHostToDevice, st));
     } else {
         d_h = const_cast<uint32_t*>(h);
         d_r = const_cast<uint16_t*>(r);
@@ -829,16 +1069,17 @@ extern "C" mhr_status mhr_tail_topk(const mhr_graph* gc, int32_t nq, const uint3
     }
 
     const double E2 = 2.0 * (g->eps32_edge + g->eps64_edge) * (1.0 + 1e-6);
-    const ScanKernel sk = pick_scan(g->dg);
+    ScanKernel sk = pick_scan(g->dg, std::min(QB, nq));
     const size_t final_smem = sizeof(BandRec) * kSortMax + (d <= kQ64Max ? sizeof(double) * d : 0);
     MHR_CUDA_TRY(cudaFuncSetAttribute(k_tail_final, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(final_smem)));
-    int per_sm = 1;
-    MHR_TRY(scan_setup(g, sk, std::min(QB, nq), &per_sm));
+    MHR_TRY(scan_setup(sk, std::min(QB, nq)));
 
     int64_t n_pairs = 0, n_surv = 0, n_band = 0, n_rescan = 0;
     double ms_scan = 0.0;
-    MHR_CUDA_TRY(cudaEventRecord(tc->ev[0], st));
-    std::vector<unsigned> hc(2 * QB), hb(QB);
+    if (stats) MHR_CUDA_TRY(cudaEventRecord(tc->ev[0], st));
+    static_assert(sizeof(unsigned) * 2 * kMaxBatch <= kPinned, "a batch's counts fit the pinned buffer");
+    unsigned* hc = reinterpret_cast<unsigned*>(tc->pinned);  // survivors, then band sizes
+    unsigned* hb = hc + QB;
     for (int c0 = 0; c0 < nq && Nc > 0; c0 += QB) {
         const int qb = std::min(QB, nq - c0);
         MHR_CUDA_TRY(cudaMemsetAsync(d_cnt, 0, 4ull * QB * 2, st));
@@ -856,7 +1097,7 @@ extern "C" mhr_status mhr_tail_topk(const mhr_graph* gc, int32_t nq, const uint3
             a.surv = d_sa;
             a.cap = capA;
             a.cnt = d_cnt;
-            MHR_TRY(launch_scan(g, sk, a, per_sm, st));
+            MHR_TRY(launch_scan(g, sk, a, st));
             k_tail_thr<<<qb, kFinalThreads, 0, st>>>(d_sa, capA, d_cnt, K, E2, d_thr);
             MHR_CUDA_TRY(cudaGetLastError());
             n_pairs += static_cast<int64_t>(qb) * M;
@@ -867,19 +1108,20 @@ extern "C" mhr_status mhr_tail_topk(const mhr_graph* gc, int32_t nq, const uint3
         a.surv = d_sb;
         a.cap = capB;
         a.cnt = cntB;
-        MHR_CUDA_TRY(cudaEventRecord(tc->ev[2], st));
-        MHR_TRY(launch_scan(g, sk, a, per_sm, st));
-        MHR_CUDA_TRY(cudaEventRecord(tc->ev[3], st));
+        if (stats) MHR_CUDA_TRY(cudaEventRecord(tc->ev[2], st));
+        MHR_TRY(launch_scan(g, sk, a, st));
+        if (stats) MHR_CUDA_TRY(cudaEventRecord(tc->ev[3], st));
         n_pairs += static_cast<int64_t>(qb) * Nc;
         k_tail_final<<<qb, kFinalThreads, final_smem, st>>>(g->dg, d_h + c0, d_r + c0, d_sb, capB, cntB, d_band, K, E2,
                                                             d_out + static_cast<int64_t>(c0) * K, d_nout + c0, d_bc);
         MHR_CUDA_TRY(cudaGetLastError());
-        MHR_CUDA_TRY(cudaMemcpyAsync(hc.data(), cntB, 4ull * qb, cudaMemcpyDeviceToHost, st));
-        MHR_CUDA_TRY(cudaMemcpyAsync(hb.data(), d_bc, 4ull * qb, cudaMemcpyDeviceToHost, st));
+        MHR_CUDA_TRY(cudaMemcpyAsync(hc, cntB, 4ull * (QB + qb), cudaMemcpyDeviceToHost, st));
         MHR_CUDA_TRY(cudaStreamSynchronize(st));
-        float ms = 0.f;
-        MHR_CUDA_TRY(cudaEventElapsedTime(&ms, tc->ev[2], tc->ev[3]));
-        ms_scan += ms;
+        if (stats) {
+            float ms = 0.f;
+            MHR_CUDA_TRY(cudaEventElapsedTime(&ms, tc->ev[2], tc->ev[3]));
+            ms_scan += ms;
+        }
         for (int i = 0; i < qb; ++i) {
             if (static_cast<int64_t>(hc[i]) <= capB) {
                 n_surv += hc[i];
@@ -903,7 +1145,7 @@ extern "C" mhr_status mhr_tail_topk(const mhr_graph* gc, int32_t nq, const uint3
             b.surv = bs;
             b.cap = Nc;
             b.cnt = bcnt;
-            MHR_TRY(launch_scan(g, sk, b, per_sm, st));
+            MHR_TRY(launch_scan(g, sk, b, st));
             k_tail_final<<<1, kFinalThreads, final_smem, st>>>(g->dg, d_h + c0 + i, d_r + c0 + i, bs, Nc, bcnt, bb, K, E2,
                                                                d_out + static_cast<int64_t>(c0 + i) * K, d_nout + c0 + i,
                                                                d_bc + i);
@@ -918,13 +1160,19 @@ extern "C" mhr_status mhr_tail_topk(const mhr_graph* gc, int32_t nq, const uint3
             ++n_rescan;
         }
     }
-    if (Nc == 0) MHR_CUDA_TRY(cudaMemsetAsync(d_nout, 0, 4ull * nq, st));
-    MHR_CUDA_TRY(cudaEventRecord(tc->ev[1], st));
+    // every batch ended with a synchronisation; wait for what came after
+    bool wait = stats != nullptr;
+    if (Nc == 0) {
+        MHR_CUDA_TRY(cudaMemsetAsync(d_nout, 0, 4ull * nq, st));
+        wait = true;
+    }
+    if (stats) MHR_CUDA_TRY(cudaEventRecord(tc->ev[1], st));
     if (mem == MHR_MEM_HOST) {
         MHR_CUDA_TRY(cudaMemcpyAsync(out, d_out, sizeof(mhr_tail) * nq * K, cudaMemcpyDeviceToHost, st));
         MHR_CUDA_TRY(cudaMemcpyAsync(n_out, d_nout, 4ull * nq, cudaMemcpyDeviceToHost, st));
+        wait = true;
     }
-    MHR_CUDA_TRY(cudaStreamSynchronize(st));
+    if (wait) MHR_CUDA_TRY(cudaStreamSynchronize(st));
     if (stats) {
         float ms_dev = 0.f;
         MHR_CUDA_TRY(cudaEventElapsedTime(&ms_dev, tc->ev[0], tc->ev[1]));

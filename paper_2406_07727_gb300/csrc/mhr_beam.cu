@@ -624,7 +624,7 @@ extern "C" mhr_status mhr_beam_paths(const mhr_graph* g, int32_t nq, const uint3
     const size_t per_query = sizeof(BeamPath) * static_cast<size_t>(2 * widest + res_cap) + 64;
     const int QB = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(nq, (int64_t(1) << 30) / per_query)));
     const double e1 = (g->eps32_edge + g->eps64_edge) * (1.0 + 1e-6);
-    const bool index = g->dg.w != nullptr && std::isfinite(e1);
+    const bool index = g->dg.w != nullptr;
     BeamPath *A = nullptr, *B = nullptr, *R = nullptr, *d_out = reinterpret_cast<BeamPath*>(out);
     uint32_t *d_s = const_cast<uint32_t*>(s), *d_t = const_cast<uint32_t*>(t), *d_left = nullptr;
     unsigned *d_nres = nullptr, *d_nleft = nullptr;

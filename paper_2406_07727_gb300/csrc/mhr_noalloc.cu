@@ -21,7 +21,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <cmath>
 #include <mutex>
 
 #include "mhr_exact.cuh"
@@ -422,7 +421,7 @@ extern "C" mhr_status mhr_topk_paths_noalloc(const mhr_graph* g, uint32_t s, uin
     uint32_t* scratch = nullptr;
     MHR_TRY(noalloc_setup(g->device, &scratch));
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (g->dg.w && std::isfinite(g->err_path))
+    if (g->dg.w)
         k_topk_noalloc<true><<<1, kNaThreads, std::max(sizeof(NoAllocSmem), sizeof(NaIndexSmem)), st>>>(
             g->dg, s, t, K, g->err_path, scratch, out, n_out);
     else

@@ -2225,15 +2225,8 @@ __global__ void __launch_bounds__(kRsWarps * 32) k_rescore(const PlanDev* __rest
         if (live) e = sum_edge(P, g, q, unit.y + lane);
         bool left = live;  // sums for the fp64 route
         if (fixed) {
-            for (int k = 0; k < m; ++k) {
-                bool ok;
-                const double x = warp_w64_fixed(g, __shfl_sync(0xffffffffu, e.h, k), __shfl_sync(0xffffffffu, e.r, k),
-                                                __shfl_sync(0xffffffffu, e.t, k), lane, &ok);
-                if (lane == k && ok) {
-                    *e.dst = x;
-                    left = false;
-                }
-            }
+            const double x = warp_w64_fixed_each(g, e.h, e.r, e.t, m, lane, left);
+            if (live && !left) *e.dst = x;
         }
         if (__any_sync(0xffffffffu, left)) {
             const double x = warp_w64_staged(g, e.h, e.r, e.t, left, stage[w], lane);

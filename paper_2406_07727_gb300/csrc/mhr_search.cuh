@@ -123,7 +123,10 @@ constexpr uint32_t kSrSegment = 2048;  // near slots gathered at a time
 constexpr uint32_t kSrSmall = 4096;  // middle edges below which no seed is worth its phases
 constexpr uint32_t kSrProbe = 98304; // middle edges worth a better threshold first (a probe costs about 60,000)
 constexpr uint32_t kSrSlice = 16384; // middle edges between threshold updates
-constexpr uint32_t kSrSample = 4096; // slots looked at for a cut or an estimate
+constexpr uint32_t kSrSample = 4096; // slots looked at for a cut
+constexpr uint32_t kSrRuns = 48;     // runs of 32 slots looked at for an estimate
+constexpr uint32_t kSrOther = 32768; // middle edges below which the other side is not estimated
+constexpr int kSrRank = 512;         // candidates up to which the K-th best is found by comparing pairs
 constexpr uint32_t kSrNone = 0xffffffffu;
 constexpr int kSrQueue = 256;        // edges that passed the far table, in shared memory
 constexpr int kSrSpillQueue = 8192;  // and past it, per block
@@ -224,12 +227,18 @@ __device__ __noinline__ float sr_cut(int sd, uint32_t want) {
     const float hi = S.maxp, lo = sm.bc[0] == 0xffffffffu ? hi : key2f(sm.bc[0]);
     const float scale = hi > lo ? 256.f / (hi - lo) : 0.f;
     uint32_t seen = 0u;
-    for (uint32_t base = 0; base < n; base += NT * stride) {
-        const uint32_t i = base + threadIdx.x;
-        seen += min(static_cast<uint32_t>(NT), n - base);
-        const float p = i < n ? S.p[i] : neg_inf();
-        if (p != neg_inf()) atomicAdd(&sm.hist[max(0, min(255, static_cast<int>((hi - p) * scale)))], 1u);
-        if (n - base <= NT * stride) break;
+    constexpr int U = 4;  // runs in flight
+    for (uint64_t base = 0; base < n; base += static_cast<uint64_t>(U) * NT * stride) {
+        float p[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t b = base + static_cast<uint64_t>(u) * NT * stride, i = b + threadIdx.x;
+            p[u] = i < n ? S.p[i] : neg_inf();
+            if (b < n) seen += static_cast<uint32_t>(min(static_cast<uint64_t>(NT), n - b));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (p[u] != neg_inf()) atomicAdd(&sm.hist[max(0, min(255, static_cast<int>((hi - p[u]) * scale)))], 1u);
     }
     const float share = static_cast<float>(want) * static_cast<float>(seen) / static_cast<float>(n);
     __syncthreads();
@@ -271,21 +280,37 @@ __device__ __noinline__ void sr_build_hash() {
     const SearchSide& F = sm.side[sm.fwd];
     const float fp = sm.far_p;
     const uint32_t n = F.n;
-    for (uint32_t i = threadIdx.x; i < n; i += NT) {
-        const float p = F.p[i];
-        if (p == neg_inf() || p < fp) continue;
-        const uint32_t v = F.col[i], k = f2key(F.w[i]);
-        if (!sr_slot_ok(sm, sm.fwd, i, v)) continue;
-        if (atomicAdd(&sm.ins, 1) >= kSrHashMax) break;
-        uint32_t h = sr_mix(v) >> 19;
-        for (;;) {
-            const uint32_t old = atomicCAS(&sm.tab[h], kSrNone, v);
-            if (old == kSrNone || old == v) {
-                atomicMax(&sm.tab[kSrHash + h], k);
-                break;
-            }
-            h = (h + 1) & (kSrHash - 1);
+    constexpr int U = 4;  // slots in flight per thread
+    for (uint32_t i0 = threadIdx.x; i0 < n; i0 += U * NT) {
+        float p[U], w[U];
+        uint32_t v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t i = i0 + u * NT;
+            const bool in = i < n && i >= i0;
+            p[u] = in ? F.p[i] : neg_inf();
+            w[u] = in ? F.w[i] : 0.f;
+            v[u] = in ? F.col[i] : 0u;
         }
+#pragma unroll 1
+        for (int u = 0; u < U; ++u) {
+            const float pu = u == 0 ? p[0] : u == 1 ? p[1] : u == 2 ? p[2] : p[3];
+            if (pu == neg_inf() || pu < fp) continue;
+            const uint32_t vu = u == 0 ? v[0] : u == 1 ? v[1] : u == 2 ? v[2] : v[3];
+            const uint32_t k = f2key(u == 0 ? w[0] : u == 1 ? w[1] : u == 2 ? w[2] : w[3]);
+            if (!sr_slot_ok(sm, sm.fwd, i0 + u * NT, vu)) continue;
+            if (atomicAdd(&sm.ins, 1) >= kSrHashMax) break;
+            uint32_t h = sr_mix(vu) >> 19;
+            for (;;) {
+                const uint32_t old = atomicCAS(&sm.tab[h], kSrNone, vu);
+                if (old == kSrNone || old == vu) {
+                    atomicMax(&sm.tab[kSrHash + h], k);
+                    break;
+                }
+                h = (h + 1) & (kSrHash - 1);
+            }
+        }
+        if (n - i0 <= U * NT) break;  // before i0 can wrap
     }
     __syncthreads();
 }
@@ -389,6 +414,26 @@ __device__ __forceinline__ uint32_t sr_row_find(const SearchSide& F, uint32_t v)
 template <int NT>
 __device__ __noinline__ void sr_select(int n) {
     SearchSmem<NT>& sm = sr_smem<NT>();
+    if (n <= kSrRank) {  // fewer barriers than the radix passes
+        for (int i = threadIdx.x; i < n; i += NT) {
+            const float mine = sm.cand[i].s32;
+            int above = 0, same = 0;
+#pragma unroll 8
+            for (int j = 0; j < n; ++j) {
+                const float x = sm.cand[j].s32;
+                above += x > mine ? 1 : 0;
+                same += x == mine ? 1 : 0;
+            }
+            if (above < sm.K && above + same >= sm.K) sm.bc[0] = f2key(mine);  // equal values, if several
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && sm.bc[0] > sm.thr_key) {
+            sm.thr_key = sm.bc[0];
+            sr_set_threshold(sm);
+        }
+        __syncthreads();
+        return;
+    }
     const uint32_t key = block_select_kth([&](int64_t i) { return f2key(sr_cand(sm, static_cast<int>(i)).s32); }, n,
                                           sm.K, sm.hist, sm.bc);
     if (threadIdx.x == 0 && key > sm.thr_key) {
@@ -495,7 +540,7 @@ __device__ __noinline__ int sr_gather(float cut, uint32_t& next) {
 }
 
 // Estimate of the near side's middle edges at or above tau, from the kept ranks of
-// up to kSrSample slots' rows (a row's edges between two known ranks are taken as
+// up to kSrRuns * 32 slots' rows (a row's edges between two known ranks are taken as
 // spread evenly between their weights; past the last one the fall of the weight
 // per factor of eight is extrapolated).  *level: about a sixteenth of them lie
 // above it.
@@ -506,19 +551,21 @@ __device__ __noinline__ float sr_estimate(float* level) {
     const SearchSide& N = sm.side[1 - sm.fwd];
     const float tau = sm.tau, top = N.maxp;
     const float scale = top > tau ? kLevels / (top - tau) : 0.f;
-    const uint32_t n = N.n, stride = (n + kSrSample - 1) / kSrSample;
+    // evenly spaced runs, a run per warp: what it costs is the chain of loads and the
+    // counters' conflicts of every slot (35,000 cycles for 4,096 slots)
+    const uint32_t runs = (N.n + 31) >> 5, stride = (runs + kSrRuns - 1) / kSrRuns, visits = (runs + stride - 1) / stride;
     // counts in units that keep every sum below 2^32
     const float unit = static_cast<float>(N.S) > 1e9f ? 1e9f / static_cast<float>(N.S) : 1.f;
     __syncthreads();
     for (int i = threadIdx.x; i < kLevels; i += NT) sm.hist[i] = 0u;
     __syncthreads();
-    uint32_t seen = 0u;
-    for (uint32_t base = 0; base < n; base += NT * stride) {
-        const uint32_t i = base + threadIdx.x;
-        seen += min(static_cast<uint32_t>(NT), n - base);
-        if (i < n && N.p[i] >= tau && N.p[i] != neg_inf()) {
-            const float wn = N.w[i];
-            const VertexRec rec = N.rec[N.col[i]];
+    for (uint32_t v = threadIdx.x >> 5; v < visits; v += NT / 32) {
+        const uint32_t i = v * stride * 32u + (threadIdx.x & 31);
+        const bool in = i < N.n;
+        const float pi = in ? N.p[i] : neg_inf(), wn = in ? N.w[i] : 0.f;
+        const uint32_t u = in ? N.col[i] : 0u;
+        if (pi >= tau && pi != neg_inf()) {
+            const VertexRec rec = N.rec[u];
             const float deg = static_cast<float>(rec.deg);
             float r0 = 0.f, f0 = __fadd_rn(wn, rec.maxw), r1 = 4.f, fall = 0.f;
 #pragma unroll 1
@@ -542,7 +589,6 @@ __device__ __noinline__ float sr_estimate(float* level) {
                 r1 *= 8.f;
             }
         }
-        if (n - base <= NT * stride) break;
     }
     __syncthreads();
     if (threadIdx.x < 32) {  // two levels per lane
@@ -554,7 +600,7 @@ __device__ __noinline__ float sr_estimate(float* level) {
         const int b = __reduce_min_sync(0xffffffffu, at);
         if (l == 0) {
             sm.cutp = scale > 0.f ? top - static_cast<float>(b + 1) / scale : tau;
-            sm.est = tot / unit * (static_cast<float>(n) / static_cast<float>(seen));
+            sm.est = tot / unit * (static_cast<float>(runs) / static_cast<float>(visits));
         }
     }
     static_assert(kLevels == 64, "two levels per lane");
@@ -846,17 +892,20 @@ __device__ void search_query(const DevGraph& g, unsigned long long heavy) {
             limit *= 8;
         }
         // side and probes
+        float last = INFINITY;
         for (int trial = 0; trial < 4 && sm.thr_key; ++trial) {
             float level, level1;
             float n = sr_estimate<NT>(&level);
-            if (n > static_cast<float>(kSrSmall) && trial < 2) {
+            if (n > static_cast<float>(kSrOther) && trial == 0) {
                 const int f0 = sm.fwd;
                 sr_face<NT>(1 - f0);
                 const float n1 = sr_estimate<NT>(&level1);
                 if (n1 < n) n = n1, level = level1;
                 else sr_face<NT>(f0);
             }
-            if (n <= static_cast<float>(kSrProbe) || n <= 4.f * static_cast<float>(spent)) break;
+            // the last probe has to have been worth its phases
+            if (n <= static_cast<float>(kSrProbe) || n <= 4.f * static_cast<float>(spent) || n > 0.6f * last) break;
+            last = n;
             const float before = sm.thr_keep;
             sr_build_far<NT>(cutf);
             if (threadIdx.x == 0) sm.cand_cnt = 0;

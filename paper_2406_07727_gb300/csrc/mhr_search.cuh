@@ -121,7 +121,7 @@ constexpr int kSrHash = 8192;        // slots of the seed's far table (vertex ->
 constexpr int kSrHashMax = 6144;     // far slots it takes
 constexpr uint32_t kSrSegment = 2048;  // near slots gathered at a time
 constexpr uint32_t kSrSmall = 4096;  // middle edges below which no seed is worth its phases
-constexpr uint32_t kSrProbe = 98304; // middle edges worth a better threshold first (a probe costs about 60,000)
+constexpr uint32_t kSrProbe = 160000; // middle edges worth a better threshold first (a probe costs about 60,000)
 constexpr uint32_t kSrSlice = 16384; // middle edges between threshold updates
 constexpr uint32_t kSrSample = 4096; // slots looked at for a cut
 constexpr uint32_t kSrRuns = 48;     // runs of 32 slots looked at for an estimate

@@ -83,12 +83,16 @@ WORKLOAD_DESCS = {
 K_OVERRIDE = 0
 WORKLOAD_DESC = WORKLOAD_DESCS[WORKLOAD]
 DATA = "synthetic: seeded R-MAT typed knowledge graph standing in for WikiKG90Mv2"
-FORM_DESC = {"plain": "plain: batched, every middle edge scored, fp32 screen + fp64 rescoring",
+FORM_DESC = {"plain": "plain: batched, threshold search over the weight index (every middle edge scored when the "
+                      "graph has none), fp32 screen + fp64 rescoring",
              "bound": "bound: plain + rows ordered by their score bound, a seed pass per query, provable "
                       "bound pruning of work items, rows and hits (identical output)",
              "chosen": "chosen: as bound, with rows ordered by the learned MLP score (trained on plain runs "
                        "over 20,000 held-out queries before timing) (identical output)"}
-# kernels per step: k_init, k_expand_v, scan x2, k_lists, k_plan, k_order_key, k_mlp_qbias,
+# kernels per step of the threshold search (graphs with a weight index): k_init, k_search, k_rescore,
+# k_merge2; queries it hands back run the join below in a conditional node
+SEARCH_KERNELS_PER_STEP = 4
+# kernels per step of the join: k_init, k_expand_v, scan x2, k_lists, k_plan, k_order_key, k_mlp_qbias,
 # k_mlp_keys, k_order_hist, scan x2, k_order_perm, scan x2, k_near, k_middle (seed),
 # k_middle, k_merge1, k_rescore, k_merge2, k_exact
 KERNELS_PER_STEP = 22
@@ -600,10 +604,11 @@ def run_beam(args):
                        "call": "mhr_beam_paths, synchronous; host arrays in and out"},
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 8 * len(S),
                     "d2h_bytes_per_step": len(S) * BEAM_K * 64 + 4 * len(S)},
-            "gpu_launches": (BEAM_H + 2) * args.steps,
+            "gpu_launches": (2 * BEAM_H + 2) * args.steps,
             "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",
                          "frac": achieved / alu_peak, "traffic": None,
-                         "kernel": "k_beam_level (all levels of a call)",
+                         "kernel": "k_beam_step / k_beam_level (all levels of a call; every out-edge of a held path "
+                                   "counts, read or not)",
                          "peak_source": f"{n_sms} SMs x 128 fp32 lanes x {sm_mhz:.0f} MHz (adds)",
                          "flops_per_call": flops},
             "clocks": clk,
@@ -782,6 +787,10 @@ def run_gpu(args):
         alg_bytes = 4 * s_near + 2 * plain_stats["hits"] + eb * g.d * n_vert
         moved_bytes = 4 * stats["edges_scanned"] + 2 * stats["hits"] + eb * g.d * n_vert
         join_avg_ms = statistics.mean(join_ms)
+        # the expansion is a part of the join's graphs only: no time of it, the threshold search ran
+        searched = expand_ms[0] == 0.0
+        if searched:  # 8 B (vertex, weight) per middle edge read, its result written
+            moved_bytes = alg_bytes = 8 * stats["edges_scanned"] + 24 * nq * K
         achieved = alg_bytes / (join_avg_ms / 1000.0) / 1e9
         peak, peak_src = measured_peaks()
         paths_per_s = plain_stats["paths"] * ws * args.steps / (elapsed_ms / 1000.0)
@@ -800,7 +809,8 @@ def run_gpu(args):
                                               else "fp32 CUDA cores"),
                        "l2": "flushed before every step (256 MiB write, excluded from the step time)",
                        "parallelism": "replicas (each rank its own queries)" if ws > 1 else "single GPU",
-                       "launch": "three CUDA graphs per step (before / join / after)",
+                       "launch": ("one CUDA graph per step" if searched
+                                  else "three CUDA graphs per step (before / join / after)"),
                        "chunk": opts.get("chunk", "library default"),
                        "tile": opts.get("tile", "library default"),
                        "autotune_ms": ({f"{'tc' if p else 'fp32'}/{c}x{t}": v
@@ -808,15 +818,18 @@ def run_gpu(args):
                                        if args.form in tuned else None)},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": 8 * nq,
                     "d2h_bytes_per_step": nq * K * 24 + 4 * nq},
-            "gpu_launches": KERNELS_PER_STEP * args.steps,
+            "gpu_launches": (SEARCH_KERNELS_PER_STEP if searched else KERNELS_PER_STEP) * args.steps,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak,
-                         "traffic": TRAFFIC_NCU.get((WORKLOAD, args.form, opts.get("chunk"), opts.get("tile"))),
+                         "traffic": (None if searched else
+                                     TRAFFIC_NCU.get((WORKLOAD, args.form, opts.get("chunk"), opts.get("tile")))),
                          "traffic_scope": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the main join launch",
-                         "kernel": "k_middle (middle join)", "peak_source": f"{peak_src} hbm_gbs",
+                         "kernel": "k_search (threshold search)" if searched else "k_middle (middle join)", "peak_source": f"{peak_src} hbm_gbs",
                          "alg_bytes_per_launch": alg_bytes, "avg_launch_ms": join_avg_ms,
                          "bytes_moved_per_launch": moved_bytes,
-                         "note": "achieved credits the plain method's algorithmic bytes (effective rate for the pruned form)"},
+                         "note": ("bytes of the middle edges the search reads (its phases wait on latency); the plain method reads "
+                                  f"{4 * s_near} bytes of them" if searched else
+                                  "achieved credits the plain method's algorithmic bytes (effective rate for the pruned form)")},
             "clocks": clk,
             "scored_paths_per_s": paths_per_s,
             "work_per_step": {"edges_scanned": stats["edges_scanned"], "edges_scanned_plain": s_near,
@@ -848,7 +861,7 @@ def run_gpu(args):
         slots = sum(f["deg_s"] + f["deg_t"] for f in fs)
         x_bytes = slots * (4 + 2) + eb * g.d * (n_vert + 2 * nq)
         x_ms = expand_ms[0]
-        result["expansion_roofline"] = {
+        result["expansion_roofline"] = None if searched else {
             "bound": "hbm", "kernel": "k_expand (hop-1 / hop-3 expansion)",
             "achieved": x_bytes / (x_ms / 1000.0) / 1e9, "peak": peak, "unit": "GB/s",
             "frac": x_bytes / (x_ms / 1000.0) / 1e9 / peak, "alg_bytes_per_launch": x_bytes,

@@ -462,7 +462,7 @@ mhr_status mhr_tail_topk(const mhr_graph* g, int32_t nq, const uint32_t* h, cons
  * and relation sequence after s (for three hops: (u, r1, v, r2, r3)).
  *   out    nq*K records (query i at out[i*K]); n_out[i] = results written
  *   mem    where s, t, out and n_out live
- *   stats  optional: edges_scanned = out-edges scored (fp32 screen),
+ *   stats  optional: edges_scanned = out-edges of the held paths (fp32 screen),
  *          rescored = extensions and results scored in fp64; ms = wall time
  * Each held path's extensions are screened in fp32 with the graph's proven
  * edge bound: only those within that bound (plus the spacing of the rounded

@@ -37,10 +37,10 @@
 // when there are queries enough for all SMs, one 1,024-thread block shortens a
 // query's phases otherwise.  Measured, whole call, against the join that reads
 // and weighs every edge of every row whose bound reaches the band: 4,096 queries
-// over 10 M vertices and 200 M edges (128 bf16 values, K = 50) 112.7 -> 4.9 ms
-// (3 % of the middle edges read); 256 over 1 M vertices and 20 M edges (256 fp32
-// values, DistMult, K = 100) 2.95 -> 0.92 ms, 64 of them (128 values, TransE)
-// 1.78 -> 0.37 ms.
+// over 10 M vertices and 200 M edges (128 bf16 values, K = 50) 112.7 -> 3.8 ms
+// (4 % of the middle edges read); 256 over 1 M vertices and 20 M edges (256 fp32
+// values, DistMult, K = 100) 3.2 -> 0.72 ms, 64 of them (128 values, TransE)
+// 1.6 -> 0.28 ms.
 //
 // A query whose candidates overflow the buffers (ties) or whose prefixes are very
 // long (fewer than K paths, a hub on both sides) is handed back (redo).

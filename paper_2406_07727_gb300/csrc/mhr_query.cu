@@ -2169,10 +2169,9 @@ __global__ void __launch_bounds__(1024) k_merge1(const PlanDev* __restrict__ P) 
 // in units of kUnit that all queries append to one list, so the kernel's warps
 // take them without looking at queries that have none.  k_merge2 adds the three
 // weights of every entry.  What bounds it: TransE, the integer issue of the
-// conversions (a warp per sum, its rows read once, whole lines); DistMult, the
-// fp64 pipe (3 d operations per sum).  256 DistMult queries, d = 256, K = 100:
-// 240 -> 181 us; 64 TransE queries, d = 128, K = 100: 51 -> 18 us;
-// 4,096 on bf16 rows, K = 50: 763 -> 310 us.
+// conversions (eight lanes per sum); DistMult, the fp64 pipe (an addition per
+// coordinate).  256 DistMult queries, d = 256, K = 100: 240 -> 107 us; 64 TransE
+// queries, d = 128, K = 100: 51 -> 16 us; 4,096 on bf16 rows, K = 50: 763 -> 230 us.
 constexpr int kRsWarps = 4;
 
 struct SumEdge {

@@ -86,8 +86,9 @@ __device__ __forceinline__ double term64(float a, float b, float c, bool transe)
 }
 
 // acc + sign * x in units of 2^-Q, sign = 1 or -1; bad is set when x is no multiple of
-// one.  |x| < 2^(53 - Q), so x = m 2^(e - 150) is m shifted left by e - 150 + Q < 30
-// places, one multiply-add into the 64-bit sum, or right by a few when it is small.
+// one.  x = m 2^(e - 150) is m shifted left by e - 150 + Q places, one multiply-add into
+// the 64-bit sum, or right by a few when it is small.  The shift stays below 30: a
+// normal x has 2^23 <= m and |x| < 2^(53 - Q); a subnormal one has e = 1 and Q <= 149.
 __device__ __forceinline__ int64_t add_fixed(int64_t acc, float x, bool minus, int Q, bool& bad) {
     const uint32_t u = __float_as_uint(x);
     const uint32_t e = (u >> 23) & 0xffu;

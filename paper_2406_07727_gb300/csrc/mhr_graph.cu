@@ -296,7 +296,9 @@ static double gam(double n, double u) { return n * u / (1.0 - n * u); }
 //   DistMult: <= g_{d+3}(2^-24) M with M = max ||w_r||_inf * max ||e||_2^2
 //           bounding sum |a b c| (Cauchy-Schwarz)
 //   the same with 2^-53 for the fp64 value, plus the two path additions.
-// Also Q of the integer route of exact weights: the sum's bound N < 2^(53 - Q).
+// Also Q of the integer route of exact weights: the sum's bound N < 2^(53 - Q), and
+// at most 149: every binary32 value is a multiple of 2^-149, and a finer unit would
+// shift subnormal coordinates past 32 bits.
 static void compute_bounds(mhr_graph* g) {
     const double u32 = std::ldexp(1.0, -24), u64 = std::ldexp(1.0, -53);
     const int d = g->dg.d;
@@ -306,7 +308,7 @@ static void compute_bounds(mhr_graph* g) {
         const double N = 2.0 * g->max_l1 + g->max_rel_l1;
         int e = 0;
         std::frexp(N, &e);  // N < 2^e
-        g->dg.qbits = 53 - std::max(-147, e + 1);
+        g->dg.qbits = std::min(149, 53 - (e + 1));
         const double gerr = std::fabs(gamma - static_cast<double>(static_cast<float>(gamma)));
         eps32 = gerr + gam(d + 4, u32) * (N + std::fabs(gamma) + 1.0);
         eps64 = gam(d + 4, u64) * (N + std::fabs(gamma) + 1.0);

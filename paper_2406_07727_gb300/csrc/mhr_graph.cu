@@ -365,7 +365,8 @@ __global__ void k_split_rel(const void* __restrict__ remb, int dtype, int64_t co
 // one (warp_rows_from).  Scoring 20 M edges of 512-byte rows (d = 128 fp32)
 // takes 1.75 ms, 5.9 TB/s of gathered tail rows through L2, which bounds it; a
 // 20-step search and a generic scorer in every lane (536 instructions per edge)
-// took 18.7 ms.  G = 0: rows that warp_score_v does not take.
+// took 18.7 ms.  G = 0: rows that warp_score_v does not take.  Every weight is summed
+// in the order of edge_w32_group with the width score_group_width gives.
 // With kout / kin the edges' order keys are also reduced to per-vertex maxima
 // (one atomic per run of lanes with the same source) and, with kout_r / kin_r,
 // to per (vertex, relation) maxima.
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(256, 3)
             }
         }
         float w;
-        if constexpr (G > 0) w = warp_score_v<G>(g, u, v, (r << 1) | 1u, lane);
+        if constexpr (G > 0) w = warp_score_v<G, G < 32>(g, u, v, (r << 1) | 1u, lane);
         else w = warp_score_any(g, u, r, v, width, lane);
         if (live && out) out[i] = w;
         if (kout) {

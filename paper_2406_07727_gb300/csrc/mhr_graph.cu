@@ -244,14 +244,14 @@ __global__ void k_fill_potentials(const int64_t* __restrict__ off, int64_t n, in
 // ---------------------------------------------------------------------------
 // norms behind the fp32 error bound
 // ---------------------------------------------------------------------------
-// Upper bounds of the largest ||x||_1 and of the largest ||x||_2^2 (or
-// ||x||_inf) over the rows: a warp per row, fp32 sums rounded up at every step
-// (at most d * 2^-23 above the exact norm, in the safe direction).  Sums in fp64
-// by one thread per row were bound by the fp64 pipe and by uncoalesced loads:
-// 1.0 ms for 1 M rows of 128 fp32 values.
+// The largest ||x||_1 and the largest ||x||_2^2 (or ||x||_inf) over the rows, in fp64.
+// Summing every row in fp64 is bound by its pipe (1.0 ms for 1 M rows of 128 fp32
+// values), so a first pass, a warp per row, sums in fp32 rounded up at every step
+// and only the rows whose sum can still be the largest are summed again.  That is a
+// handful of rows, or, when all rows have the same norm, every one at the old cost.
 __global__ void __launch_bounds__(256) k_row_norms(const void* __restrict__ tab, int dtype, int64_t rows, int d,
-                                                   unsigned long long* __restrict__ max_l1,
-                                                   unsigned long long* __restrict__ max_aux, int aux_is_inf) {
+                                                   float2* __restrict__ sums, unsigned* __restrict__ top,
+                                                   int aux_is_inf) {
     __shared__ float s1[8], s2[8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     float m1 = 0.f, m2 = 0.f;
@@ -268,6 +268,7 @@ __global__ void __launch_bounds__(256) k_row_norms(const void* __restrict__ tab,
             const float y = __shfl_xor_sync(0xffffffffu, aux, o);
             aux = aux_is_inf ? fmaxf(aux, y) : __fadd_ru(aux, y);
         }
+        if (lane == 0) sums[r] = make_float2(l1, aux);
         m1 = fmaxf(m1, l1);
         m2 = fmaxf(m2, aux);
     }
@@ -281,9 +282,36 @@ __global__ void __launch_bounds__(256) k_row_norms(const void* __restrict__ tab,
             m1 = fmaxf(m1, s1[w]);
             m2 = fmaxf(m2, s2[w]);
         }
+        // non-negative floats compare like their bit patterns
+        atomicMax(top + 0, __float_as_uint(m1));
+        atomicMax(top + 1, __float_as_uint(m2));
+    }
+}
+
+// The candidates of k_row_norms in fp64, j = 0 .. d-1, a thread per row.  A rounded-up
+// sum is at most d / 32 + 6 steps of 2^-23 above the exact one, and 2^-149 more per
+// element whose square underflows.
+__global__ void __launch_bounds__(256) k_row_norms64(const void* __restrict__ tab, int dtype, int64_t rows, int d,
+                                                     const float2* __restrict__ sums, const unsigned* __restrict__ top,
+                                                     unsigned long long* __restrict__ max_l1,
+                                                     unsigned long long* __restrict__ max_aux, int aux_is_inf) {
+    const double keep = 1.0 - (d / 32 + 8) * 0x1p-23, tiny = d * 0x1p-149;
+    const double lo1 = static_cast<double>(__uint_as_float(top[0])) * keep - tiny;
+    const double lo2 = static_cast<double>(__uint_as_float(top[1])) * keep - tiny;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t r = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; r < rows; r += stride) {
+        const float2 s = sums[r];
+        if (!(s.x >= lo1 || s.y >= lo2)) continue;
+        double l1 = 0.0, aux = 0.0;
+#pragma unroll 8
+        for (int j = 0; j < d; ++j) {
+            const double x = fabs(static_cast<double>(emb_f32(tab, dtype, r, d, j)));
+            l1 += x;
+            aux = aux_is_inf ? fmax(aux, x) : aux + x * x;
+        }
         // non-negative doubles compare like their bit patterns
-        atomicMax(max_l1, static_cast<unsigned long long>(__double_as_longlong(static_cast<double>(m1))));
-        atomicMax(max_aux, static_cast<unsigned long long>(__double_as_longlong(static_cast<double>(m2))));
+        atomicMax(max_l1, static_cast<unsigned long long>(__double_as_longlong(l1)));
+        atomicMax(max_aux, static_cast<unsigned long long>(__double_as_longlong(aux)));
     }
 }
 
@@ -811,12 +839,18 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
     MHR_CUDA_TRY(cudaMemcpyAsync(g->h_roff.data(), roff, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, st));
 
     // --- norms
-    unsigned long long* mx;
-    MHR_CUDA_TRY(tmp.alloc(&mx, sizeof(unsigned long long) * 4));
-    MHR_CUDA_TRY(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * 4, st));
-    k_row_norms<<<grid, 256, 0, st>>>(vemb, desc->emb_dtype, n, d, mx + 0, mx + 1, 0);
-    k_row_norms<<<std::max(1, std::min(grid, (R + 7) / 8)), 256, 0, st>>>(remb, desc->emb_dtype, R, d,
-                                                                               mx + 2, mx + 3, 1);
+    unsigned long long* mx;  // four maxima in fp64, then the four of the first pass in fp32
+    MHR_CUDA_TRY(tmp.alloc(&mx, sizeof(unsigned long long) * 6));
+    MHR_CUDA_TRY(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * 6, st));
+    unsigned* top = reinterpret_cast<unsigned*>(mx + 4);
+    float2* sums = reinterpret_cast<float2*>(src);  // the sort is done with its scratch
+    const int64_t most = std::max<int64_t>(n, R);
+    if (!src || 5 * E < 2 * most) MHR_CUDA_TRY(tmp.alloc(&sums, sizeof(float2) * most));
+    const int rgrid = std::max(1, std::min(grid, (R + 7) / 8));
+    k_row_norms<<<grid, 256, 0, st>>>(vemb, desc->emb_dtype, n, d, sums, top, 0);
+    k_row_norms64<<<grid, 256, 0, st>>>(vemb, desc->emb_dtype, n, d, sums, top, mx + 0, mx + 1, 0);
+    k_row_norms<<<rgrid, 256, 0, st>>>(remb, desc->emb_dtype, R, d, sums, top + 2, 1);
+    k_row_norms64<<<rgrid, 256, 0, st>>>(remb, desc->emb_dtype, R, d, sums, top + 2, mx + 2, mx + 3, 1);
     MHR_CUDA_TRY(cudaGetLastError());
     unsigned long long hm[4];
     MHR_CUDA_TRY(cudaMemcpyAsync(hm, mx, sizeof hm, cudaMemcpyDeviceToHost, st));

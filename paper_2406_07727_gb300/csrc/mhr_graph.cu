@@ -623,6 +623,11 @@ struct IndexArrays {
     unsigned long long *sout, *sin;
 };
 
+// bytes of the split relation table
+size_t split_bytes(const mhr_graph* g) {
+    return g->fn == MHR_SCORE_DISTMULT ? sizeof(uint16_t) * 2 * static_cast<size_t>(g->dg.R) * g->dg.d : 0;
+}
+
 // The index is kept when it fits: within the graph's memory cap, and within
 // half of the device memory that is free once the graph itself is resident (the
 // rest stays for query plans).  A graph without one runs the joins that weigh
@@ -633,8 +638,9 @@ void alloc_index(mhr_graph* g, int64_t n, int64_t E, IndexArrays* ix) {
     const size_t e2 = round(sizeof(uint16_t) * E), e4 = round(sizeof(uint32_t) * E), e8 = round(sizeof(uint2) * E),
                  n8 = round(sizeof(unsigned long long) * n), nr = round(sizeof(VertexRec) * n);
     const size_t total = 2 * (e2 + 2 * e4 + e8 + n8 + nr);
-    // still to come: the reverse adjacency, and (released later) the sort's scratch
-    const size_t later = static_cast<size_t>(E) * 6 + static_cast<size_t>(n) * 8;
+    // still to come: the reverse adjacency and DistMult's split relation table, and
+    // (released later) a list of the sort
+    const size_t later = static_cast<size_t>(E) * 6 + sizeof(int64_t) * (n + 1) + split_bytes(g);
     if (g->memory_cap && g->alloc_bytes + total + later > g->memory_cap) return;
     size_t avail = 0, all = 0;
     if (cudaMemGetInfo(&avail, &all) != cudaSuccess || avail < later + static_cast<size_t>(E) * 4 ||
@@ -885,7 +891,7 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
     compute_bounds(g);
     if (g->fn == MHR_SCORE_DISTMULT) {
         const int64_t cnt = static_cast<int64_t>(R) * d;
-        MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&g->wsplit), sizeof(uint16_t) * 2 * cnt));
+        MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&g->wsplit), split_bytes(g)));
         k_split_rel<<<std::max(1, std::min(grid, static_cast<int>((cnt + 255) / 256))), 256, 0, st>>>(
             remb, desc->emb_dtype, cnt, g->wsplit, g->wsplit + cnt);
         MHR_CUDA_TRY(cudaGetLastError());

@@ -136,8 +136,8 @@ static_assert(sizeof(float) * kTcRows * 65 <= sizeof(DwSmem::A), "the tile of dW
 
 __global__ void __launch_bounds__(kTcThreads, 2)
     k_mlp_bwd_tc(const float* __restrict__ w2, const float* __restrict__ y, const float* __restrict__ tgt,
-                 const float* __restrict__ z1, const uint16_t* __restrict__ X, int64_t n, float* __restrict__ part,
-                 float* __restrict__ loss) {
+                 const float* __restrict__ z1, bool z_vec, const uint16_t* __restrict__ X, int64_t n,
+                 float* __restrict__ part, float* __restrict__ loss) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     DwSmem& sm = *reinterpret_cast<DwSmem*>(smem_raw);
     const int i0 = blockIdx.x * 64, o0 = blockIdx.y * kTcRows;
@@ -189,9 +189,14 @@ __global__ void __launch_bounds__(kTcThreads, 2)
                 const int64_t row = r0 + rg * 8 + j;
                 float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
                 if (row < n) {
-                    const float4* src = reinterpret_cast<const float4*>(z1 + row * kMlpHid + o0 + blk * 8);
-                    a = __ldg(src);
-                    b = __ldg(src + 1);
+                    const float* z = z1 + row * kMlpHid + o0 + blk * 8;
+                    if (z_vec) {
+                        a = __ldg(reinterpret_cast<const float4*>(z));
+                        b = __ldg(reinterpret_cast<const float4*>(z) + 1);
+                    } else {
+                        a = make_float4(__ldg(z), __ldg(z + 1), __ldg(z + 2), __ldg(z + 3));
+                        b = make_float4(__ldg(z + 4), __ldg(z + 5), __ldg(z + 6), __ldg(z + 7));
+                    }
                 }
                 v[j][0] = a.x; v[j][1] = a.y; v[j][2] = a.z; v[j][3] = a.w;
                 v[j][4] = b.x; v[j][5] = b.y; v[j][6] = b.z; v[j][7] = b.w;
@@ -437,10 +442,11 @@ extern "C" mhr_status mhr_mlp_backward(const mhr_mlp* m, const uint16_t* X, int6
     // slice's gradients in the scratch (258 rows of it hold one slice).
     const int64_t fit = n * kMlpHid / kDwPart, fill = std::max(1, 2 * sms / 8);
     const int slices = static_cast<int>(std::max<int64_t>(1, std::min({fit, fill, (n + kDwRows - 1) / kDwRows})));
+    const bool z_vec = reinterpret_cast<uintptr_t>(z1) % 16 == 0;  // a caller's z1 is aligned to a float
     MHR_CUDA_TRY(cudaFuncSetAttribute(k_mlp_bwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       static_cast<int>(sizeof(DwSmem))));
     k_mlp_bwd_tc<<<dim3(kMlpIn / 64, kMlpHid / kTcRows, slices), kTcThreads, sizeof(DwSmem), st>>>(
-        m->w2, y, target, z1, X, n, slices > 1 ? work : grads, loss);
+        m->w2, y, target, z1, z_vec, X, n, slices > 1 ? work : grads, loss);
     if (slices > 1) k_mlp_bwd_sum<<<(kMlpParams + 256) / 256, 256, 0, st>>>(work, slices, n, grads, loss);
     MHR_CUDA_TRY(cudaGetLastError());
     return MHR_OK;

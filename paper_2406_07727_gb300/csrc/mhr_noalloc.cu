@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kNaThreads) k_topk_noalloc(const __grid_consta
             sm.cand_cnt = 0;
         }
         __syncthreads();
-        search_query<kNaThreads>(g, ~0ull);  // the walk would read no fewer edges
+        search_query<kNaThreads>(g, ~0ull, ~0ull);  // the walk would read no fewer edges
         __syncthreads();
         const bool redo = sm.redo != 0 || sm.cand_cnt > kNaCand;
         __syncthreads();

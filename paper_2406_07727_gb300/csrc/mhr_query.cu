@@ -2024,7 +2024,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(const PlanDev* __restr
             sm.cand_cnt = 0;
         }
         __syncthreads();
-        if (valid) search_query<NT>(g, static_cast<unsigned long long>(P->heavy));
+        if (valid)
+            search_query<NT>(g, static_cast<unsigned long long>(P->heavy), static_cast<unsigned long long>(P->alone));
         __syncthreads();
         const int m = sm.cand_cnt;
         const bool redo = valid && (sm.redo || m > band_cap);
@@ -3157,6 +3158,11 @@ static mhr_status run_batch(mhr_graph* G, int nq, const uint32_t* hS, const uint
         p->h.prune = 1;
         if (p->h.order == 0) p->h.order = 1;
         p->h.heavy = int64_t(1) << 22;
+        // Without a threshold (fewer than K paths found) every middle edge has to be
+        // read.  One block reads 1.7 G edges/s, the join 73 G edges/s after 0.2 ms of
+        // launches: a lone query is better off there past 2^18 edges, and a batch keeps
+        // its blocks busy for longer.
+        p->h.alone = std::min<int64_t>(p->h.heavy, (int64_t(1) << 18) + (int64_t(nq) << 14));
         // largest rows first (by powers of two), so that no long query starts last
         uint32_t* ord = reinterpret_cast<uint32_t*>(p->pin + L.off_ord);
         uint32_t first[65] = {0};

@@ -96,7 +96,8 @@ struct PlanDev {
     const uint32_t* qord;  // [nq] queries, largest rows first
     Cand* spill;           // [search grid x kSrSpill] candidates past a block's shared buffer
     SrPass* spill_queue;   // [search grid x kSrSpillQueue] edges to look up past its shared queue
-    int64_t heavy;         // middle edges after which a query is handed back
+    int64_t heavy;         // middle edges after which a query is handed back,
+    int64_t alone;         // and while it has no threshold
     MlpDev mlp;            // order 2 weights
     int64_t nhist;        // nq * 256 order buckets
     int64_t item_cap;     // capacity of item_ub

@@ -43,7 +43,8 @@
 // 1.6 -> 0.28 ms.
 //
 // A query whose candidates overflow the buffers (ties) or whose prefixes are very
-// long (fewer than K paths, a hub on both sides) is handed back (redo).
+// long (fewer than K paths, a hub on both sides) is handed back (redo): one without a
+// threshold after `alone` middle edges, which the join's blocks read together sooner.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -675,6 +676,7 @@ __device__ __noinline__ unsigned long long sr_scan(bool probe, uint32_t limit, f
             block_excl_scan<unsigned long long>(ne, sm.red, &total);
             read += total;
             if (read > budget) {  // block-uniform
+                read -= total;
                 if (!SEED && !probe && threadIdx.x == 0) sm.redo = 1;
                 next = N.n;
                 break;
@@ -821,12 +823,30 @@ __device__ __noinline__ unsigned long long sr_scan(bool probe, uint32_t limit, f
     return read;
 }
 
+// middle edges of the near slots that may lie on a path
+template <int NT>
+__device__ __noinline__ unsigned long long sr_open_edges() {
+    SearchSmem<NT>& sm = sr_smem<NT>();
+    const SearchSide& N = sm.side[1 - sm.fwd];
+    unsigned long long mine = 0ull;
+#pragma unroll 4
+    for (uint32_t base = 0; base < N.n; base += NT) {
+        const uint32_t i = base + threadIdx.x;
+        if (i >= N.n) break;
+        const uint32_t u = N.col[i];
+        if (sr_slot_ok(sm, 1 - sm.fwd, i, u)) mine += N.rec[u].deg;
+        if (N.n - base <= NT) break;  // before base can wrap
+    }
+    return block_sum<unsigned long long>(mine, sm.red);
+}
+
 // The whole search of the query described by sm.s, t, K, two_err, cons, part_*,
 // spill and cap.  Afterwards sm.redo tells whether the query is handed back;
 // otherwise sr_cand(0 .. sm.cand_cnt) are all paths that can be among the K
-// best.  heavy: middle edges after which the query is handed back.
+// best.  heavy: middle edges after which the query is handed back; alone: the same
+// while no threshold is known.
 template <int NT>
-__device__ void search_query(const DevGraph& g, unsigned long long heavy) {
+__device__ void search_query(const DevGraph& g, unsigned long long heavy, unsigned long long alone) {
     SearchSmem<NT>& sm = sr_smem<NT>();
     if (threadIdx.x < 2) {
         SearchSide& S = sm.side[threadIdx.x];
@@ -863,6 +883,19 @@ __device__ void search_query(const DevGraph& g, unsigned long long heavy) {
     sr_face<NT>(sm.side[0].S <= sm.side[1].S ? 1 : 0);
     const unsigned long long S_near = sm.side[1 - sm.fwd].S;
     if (threadIdx.x == 0) sm.near_edges = S_near;
+    unsigned long long S_open = S_near;  // of slots that may lie on a path
+    if (S_near > kSrSmall && (sm.cons || sm.part_count > 1)) {
+        S_open = sr_open_edges<NT>();
+        // Constraints past the near slots are tested hit by hit: seeds and thresholds
+        // fail on most, and with many edges the join's blocks are faster together
+        // (middle relation and one type allowed, two hubs, 5 M edges, K = 1,000: 1.87 ms
+        // here, 0.42 ms there; 256 such queries 7.7 and 6.3 ms)
+        if (sm.cons && S_open > alone) {
+            if (threadIdx.x == 0) sm.redo = 1;
+            __syncthreads();
+            return;
+        }
+    }
     if (S_near > kSrSmall) {
         // seed: rows and edges per row grow until K paths are found
         const int nsd = 1 - sm.fwd, fsd = sm.fwd;
@@ -871,7 +904,7 @@ __device__ void search_query(const DevGraph& g, unsigned long long heavy) {
         if (threadIdx.x == 0) sm.far_p = cutf;
         __syncthreads();
         sr_build_hash<NT>();
-        unsigned long long spent = 0;
+        unsigned long long spent = 0, left = alone;
         for (int trial = 0; trial < 4; ++trial) {
             const float cut = sr_cut<NT>(nsd, rows);
             __syncthreads();
@@ -880,16 +913,28 @@ __device__ void search_query(const DevGraph& g, unsigned long long heavy) {
                 sm.cand_cnt = 0;
             }
             __syncthreads();
-            spent = sr_scan<NT, true>(false, limit, neg_inf(), static_cast<unsigned long long>(rows) * limit * 2);
+            spent = sr_scan<NT, true>(false, limit, neg_inf(),
+                                      min(left, static_cast<unsigned long long>(rows) * limit * 2));
+            left -= spent;
             const int nc = min(sm.cand_cnt, sm.cap);
             __syncthreads();
             if (nc >= sm.K) {
                 sr_select<NT>(nc);
                 break;
             }
-            if (spent * 4 > S_near * 3) break;  // nearly all of it read
+            // half of it read, or too few paths for a threshold at this rate
+            if (spent * 2 > S_open) break;
+            if (spent >= kSrSmall && 2ull * nc * S_open < spent * static_cast<unsigned long long>(sm.K)) break;
             rows *= 4;
             limit *= 8;
+        }
+        if (!sm.thr_key && S_open > alone) {
+            if (threadIdx.x == 0) {
+                sm.cand_cnt = 0;
+                sm.redo = 1;
+            }
+            __syncthreads();
+            return;
         }
         // side and probes
         float last = INFINITY;

@@ -18,9 +18,9 @@
 //      survivor list;
 //   4. per query (k_tail_final): the exact K-th best fp32 survivor score by a
 //      radix select, the band of survivors within twice the error bound of it
-//      rescored in fp64 in the canonical operation order (TransE a warp per member
-//      in integers; otherwise one member per thread, e_h + w_r formed once in fp64
-//      in shared memory), and the K best of the band put in order, a short band by
+//      rescored in fp64 in the canonical operation order (TransE in integers by
+//      eight lanes per member; otherwise one member per thread, e_h + w_r formed once
+//      in fp64 in shared memory), and the K best of the band put in order, a short band by
 //      comparing every pair (64 queries, K = 50: 33 -> 16 us).
 //
 // Exactness: |S32 - w64| <= E = eps32 + eps64 for every candidate (the bound of
@@ -653,14 +653,15 @@ __global__ void __launch_bounds__(kFinalThreads)
     double lo = -INFINITY;
     if (n > K) lo = __dsub_rd(static_cast<double>(select_kth_score(a, n, K, sm)), E2);
     if (threadIdx.x == 0) sm.count = 0u;
-    if (shared_q) {
-        for (int j = threadIdx.x; j < g.d; j += blockDim.x) {
-            const double e = static_cast<double>(emb_f32(g.vemb, g.dtype, hq, g.d, j));
-            const double w = static_cast<double>(emb_f32(g.remb, g.dtype, rq, g.d, j));
-            q64[j] = transe ? __dadd_rn(e, w) : __dmul_rn(e, w);
-        }
+    bool bad = false;  // the query's own rows are no multiples of the integers' unit
+    for (int j = threadIdx.x; j < g.d; j += blockDim.x) {
+        const float e = emb_f32(g.vemb, g.dtype, hq, g.d, j), w = emb_f32(g.remb, g.dtype, rq, g.d, j);
+        if (transe) add_fixed(add_fixed(0, e, false, g.qbits, bad), w, false, g.qbits, bad);
+        if (!shared_q) continue;
+        const double e64 = static_cast<double>(e), w64 = static_cast<double>(w);
+        q64[j] = transe ? __dadd_rn(e64, w64) : __dmul_rn(e64, w64);
     }
-    __syncthreads();
+    const bool whole = !__syncthreads_or(bad);
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
         const SurvRec x = a[i];
         if (static_cast<double>(x.s) >= lo) {
@@ -670,29 +671,36 @@ __global__ void __launch_bounds__(kFinalThreads)
     }
     __syncthreads();
     const unsigned nb = sm.count;
-    // fp64 rescoring: TransE a warp per member, in integers; members the integers do
-    // not hold, and DistMult, one per thread over dense warps
+    // fp64 rescoring.  TransE in integers, eight lanes per member and four members at a
+    // time; a lane's share of a row is 32 coordinates' steps, so short rows of many
+    // members, members the integers do not hold and DistMult go one per thread, over
+    // dense warps.  200,000 members of 4 values: 2.1 ms by threads, 13 ms by a warp per
+    // member; the whole call for 1,000 members: d = 16 157 and 155 us, 48 180 and 176, 64
+    // 194 and 172, 128 252 and 189; for 40,000: d = 16 1.05 and 1.21 ms, 32 1.59 and
+    // 1.20, 48 2.14 and 2.47, 64 2.68 and 1.85, 128 4.86 and 3.09; up to 128 members
+    // the integers are never slower (threads, integers).
+    const bool fixed = transe && whole && (nb <= 128u || g.d >= 64 || g.d % 32 == 0);
     __syncthreads();  // everyone has nb
     if (threadIdx.x == 0) sm.count = 0u;
     __syncthreads();
-    if (transe) {
+    if (fixed) {
         const int lane = threadIdx.x & 31;
-#pragma unroll 2
-        for (unsigned p = threadIdx.x >> 5; p < nb; p += kFinalThreads / 32) {
-            const uint32_t v = b[p].v;
-            bool ok;
-            const double w = warp_w64_fixed(g, hq, rq, v, lane, &ok);
-            if (lane == 0) {
-                b[p] = BandRec{w, v, ok ? 0u : 1u};
-                if (!ok) sm.count = 1u;
-            }
+        constexpr unsigned W = kFinalThreads / 32;
+        const unsigned per = min(32u, (nb + 4 * W - 1) / (4 * W) * 4u);  // members of a warp's step
+        for (unsigned b0 = (threadIdx.x >> 5) * per; b0 < nb; b0 += per * W) {
+            const int m = static_cast<int>(min(per, nb - b0));
+            bool left = lane < m;
+            const uint32_t v = left ? b[b0 + lane].v : 0u;
+            const double w = warp_w64_fixed_each(g, hq, rq, v, m, lane, left);
+            if (lane < m) b[b0 + lane] = BandRec{w, v, left ? 1u : 0u};
+            if (left) sm.count = 1u;
         }
         __syncthreads();
     }
-    if (!transe || sm.count) {
+    if (!fixed || sm.count) {
         for (unsigned p = threadIdx.x; p < nb; p += blockDim.x) {
             const uint32_t v = b[p].v;
-            if (transe && b[p].pad == 0u) continue;
+            if (fixed && b[p].pad == 0u) continue;
             double w;
             if (!shared_q) w = edge_w64(g, hq, rq, v);
             else if (transe) w = rescore_row<true>(g, q64, v);

@@ -395,25 +395,30 @@ __global__ void k_split_rel(const void* __restrict__ remb, int dtype, int64_t co
 // 20-step search and a generic scorer in every lane (536 instructions per edge)
 // took 18.7 ms.  G = 0: rows that warp_score_v does not take.  Every weight is summed
 // in the order of edge_w32_group with the width score_group_width gives.
+// FEW: a warp takes `per` < 32 edges at a time, when 32 would leave warps idle.
 // With kout / kin the edges' order keys are also reduced to per-vertex maxima
 // (one atomic per run of lanes with the same source) and, with kout_r / kin_r,
 // to per (vertex, relation) maxima.
-template <int G>
-__global__ void __launch_bounds__(256, 3)
+// Resident blocks per SM: three with four rounds of rows in flight, eight for the one
+// row in flight of G = 0 (400,000 edges of 513 fp32 values: 0.69 ms at three, 0.44).
+constexpr int edge_blocks(int G) { return G ? 3 : 8; }
+template <int G, bool FEW>
+__global__ void __launch_bounds__(256, edge_blocks(G))
     k_edge_w32(DevGraph g, const uint32_t* __restrict__ src, const uint16_t* __restrict__ rel,
-               const uint32_t* __restrict__ dst, int64_t m, int width, float* __restrict__ out,
+               const uint32_t* __restrict__ dst, int64_t m, int per, int width, float* __restrict__ out,
                uint32_t* __restrict__ kout, uint32_t* __restrict__ kin, uint32_t* __restrict__ kout_r,
                uint32_t* __restrict__ kin_r) {
+    if (!FEW) per = 32;
     const int lane = threadIdx.x & 31;
     const int64_t warp_id = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
     const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    const int64_t steps = (m + 31) >> 5;
+    const int64_t steps = (m + per - 1) / per;
     const int64_t s0 = steps * warp_id / nwarps, s1 = steps * (warp_id + 1) / nwarps;
     if (s0 >= s1) return;  // warp-uniform
-    int64_t row = src ? 0 : warp_row_search(g.off, g.n, s0 * 32, lane);
+    int64_t row = src ? 0 : warp_row_search(g.off, g.n, s0 * per, lane);
     for (int64_t st = s0; st < s1; ++st) {
-        const int64_t i = st * 32 + lane;
-        const bool live = i < m;
+        const int64_t i = st * per + lane;
+        const bool live = (!FEW || lane < per) && i < m;
         uint32_t u = 0, r = 0, v = 0;  // dead lanes score vertex 0's rows
         if (src) {
             if (live) {
@@ -423,7 +428,7 @@ __global__ void __launch_bounds__(256, 3)
             }
         } else {
             const int64_t mine = warp_rows_from(g.off, g.n, row, min(i, m - 1), lane);
-            row = __shfl_sync(0xffffffffu, mine, 31);
+            row = __shfl_sync(0xffffffffu, mine, per - 1);
             if (live) {
                 u = static_cast<uint32_t>(mine);
                 r = g.rel[i];
@@ -431,7 +436,7 @@ __global__ void __launch_bounds__(256, 3)
             }
         }
         float w;
-        if constexpr (G > 0) w = warp_score_v<G, G < 32>(g, u, v, (r << 1) | 1u, lane);
+        if constexpr (G > 0) w = warp_score_v<G, G < 32, FEW>(g, u, v, (r << 1) | 1u, lane, per);
         else w = warp_score_any(g, u, r, v, width, lane);
         if (live && out) out[i] = w;
         if (kout) {
@@ -450,28 +455,56 @@ __global__ void __launch_bounds__(256, 3)
     }
 }
 
+// Triples whose rows warp_score_v does not take: a group of `width` lanes per triple,
+// all resident warps at once.  A warp of the kernel above goes through 32 of them in
+// turn: 512,000 triples of 513 fp32 values 0.56 ms, here 0.28; 100 of them 122 us, 30.
+__global__ void __launch_bounds__(256) k_triple_w32(DevGraph g, const uint32_t* __restrict__ src,
+                                                    const uint16_t* __restrict__ rel, const uint32_t* __restrict__ dst,
+                                                    int64_t m, int width, float* __restrict__ out) {
+    const int sub = threadIdx.x & (width - 1), per = blockDim.x / width;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * per;
+    const int64_t ends = (m + per - 1) / per * per;  // every lane of a warp takes the same steps
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * per + threadIdx.x / width; i < ends; i += stride) {
+        const int64_t e = min(i, m - 1);
+        const float w = edge_w32_group(g, src[e], rel[e], dst[e], sub, width);
+        if (sub == 0 && i < m) out[i] = w;
+    }
+}
+
 // launch of k_edge_w32 with the graph's scorer
+using EdgeKernel = void (*)(DevGraph, const uint32_t*, const uint16_t*, const uint32_t*, int64_t, int, int, float*,
+                            uint32_t*, uint32_t*, uint32_t*, uint32_t*);
+template <bool FEW>
+static EdgeKernel edge_kernel(int G) {
+    switch (G) {
+        case 1: return k_edge_w32<1, FEW>;
+        case 2: return k_edge_w32<2, FEW>;
+        case 4: return k_edge_w32<4, FEW>;
+        case 8: return k_edge_w32<8, FEW>;
+        case 16: return k_edge_w32<16, FEW>;
+        default: return k_edge_w32<32, FEW>;
+    }
+}
+
 static cudaError_t launch_edge_w32(const DevGraph& g, const uint32_t* src, const uint16_t* rel, const uint32_t* dst,
                                    int64_t m, float* out, uint32_t* kout, uint32_t* kin, uint32_t* kout_r,
                                    uint32_t* kin_r, int sms, cudaStream_t st) {
     if (m <= 0) return cudaSuccess;
-    const int G = hit_group_width(g.d, g.dtype, 2);
-    void (*fn)(DevGraph, const uint32_t*, const uint16_t*, const uint32_t*, int64_t, int, float*, uint32_t*, uint32_t*,
-               uint32_t*, uint32_t*) = k_edge_w32<0>;
-    if (score_vec2(g, G)) {
-        switch (G) {
-            case 1: fn = k_edge_w32<1>; break;
-            case 2: fn = k_edge_w32<2>; break;
-            case 4: fn = k_edge_w32<4>; break;
-            case 8: fn = k_edge_w32<8>; break;
-            case 16: fn = k_edge_w32<16>; break;
-            default: fn = k_edge_w32<32>; break;
-        }
+    const int G = hit_group_width(g.d, g.dtype, 2), width = score_group_width(g.d, g.dtype);
+    const bool vec = score_vec2(g, G);
+    if (!vec && src && !kout) {
+        const int64_t blocks = std::min<int64_t>(static_cast<int64_t>(sms) * 8, (m * width + 255) / 256);
+        k_triple_w32<<<static_cast<unsigned>(blocks), 256, 0, st>>>(g, src, rel, dst, m, width, out);
+        return cudaGetLastError();
     }
-    // one resident wave (three blocks per SM by the launch bounds)
-    const int64_t blocks = std::min<int64_t>(static_cast<int64_t>(sms) * 3, (m + 255) / 256);
-    fn<<<static_cast<unsigned>(blocks), 256, 0, st>>>(g, src, rel, dst, m, score_group_width(g.d, g.dtype), out, kout,
-                                                     kin, kout_r, kin_r);
+    // one resident wave, and steps of as many edges as still give every warp one
+    const int64_t wave = static_cast<int64_t>(sms) * edge_blocks(vec ? G : 0);
+    const int least = vec ? 32 / G * std::min(G, kScoreRounds) : 32;  // edges a warp scores together
+    int per = 32;
+    while (per > least && (m + per - 1) / per < wave * 8) per >>= 1;
+    const EdgeKernel fn = !vec ? k_edge_w32<0, false> : (per < 32 ? edge_kernel<true>(G) : edge_kernel<false>(G));
+    const int64_t blocks = std::min<int64_t>(wave, ((m + per - 1) / per + 7) / 8);
+    fn<<<static_cast<unsigned>(blocks), 256, 0, st>>>(g, src, rel, dst, m, per, width, out, kout, kin, kout_r, kin_r);
     return cudaGetLastError();
 }
 
@@ -503,23 +536,24 @@ __global__ void k_edge_scores64(DevGraph g, const uint32_t* __restrict__ src,
 // coordinate: for 2M edges of 128 fp32 values 2.82 ms, now 0.82 ms (TransE) and 1.16
 // ms (DistMult); of 16 values 0.36 ms against 0.23 and 0.26; of 8 values 0.19 ms both.
 // Shorter rows than kEdge64Warp keep it: a step covers 32 coordinates, filled or not.
+// As above, `per` is less than 32 (a multiple of four) for few edges.
 constexpr int kEdge64Warps = 4;
 constexpr int kEdge64Warp = 16;
 __global__ void __launch_bounds__(kEdge64Warps * 32) k_edge_scores64_warp(DevGraph g, const uint32_t* __restrict__ src,
                                                                          const uint16_t* __restrict__ rel,
                                                                          const uint32_t* __restrict__ dst, int64_t m,
-                                                                         double* __restrict__ out) {
+                                                                         int per, double* __restrict__ out) {
     __shared__ double stage[kEdge64Warps][32 * 33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t warp_id = blockIdx.x * static_cast<int64_t>(kEdge64Warps) + w;
     const int64_t nwarps = static_cast<int64_t>(gridDim.x) * kEdge64Warps;
-    const int64_t steps = (m + 31) >> 5;
+    const int64_t steps = (m + per - 1) / per;
     const int64_t s0 = steps * warp_id / nwarps, s1 = steps * (warp_id + 1) / nwarps;
     if (s0 >= s1) return;  // warp-uniform; no block-wide step below
-    int64_t row = src ? 0 : warp_row_search(g.off, g.n, s0 * 32, lane);
+    int64_t row = src ? 0 : warp_row_search(g.off, g.n, s0 * per, lane);
     for (int64_t st = s0; st < s1; ++st) {
-        const int64_t i = st * 32 + lane;
-        const bool live = i < m;
+        const int64_t i = st * per + lane;
+        const bool live = lane < per && i < m;
         uint32_t u = 0, r = 0, v = 0;
         if (src) {
             if (live) {
@@ -529,7 +563,7 @@ __global__ void __launch_bounds__(kEdge64Warps * 32) k_edge_scores64_warp(DevGra
             }
         } else {
             const int64_t mine = warp_rows_from(g.off, g.n, row, min(i, m - 1), lane);
-            row = __shfl_sync(0xffffffffu, mine, 31);
+            row = __shfl_sync(0xffffffffu, mine, per - 1);
             if (live) {
                 u = static_cast<uint32_t>(mine);
                 r = g.rel[i];
@@ -539,7 +573,7 @@ __global__ void __launch_bounds__(kEdge64Warps * 32) k_edge_scores64_warp(DevGra
         double mine = 0.0;
         bool left = live;
         if (g.fn == MHR_SCORE_TRANSE_L1) {
-            const int n = static_cast<int>(min(static_cast<int64_t>(32), m - st * 32));
+            const int n = static_cast<int>(min(static_cast<int64_t>(per), m - st * per));
             mine = warp_w64_fixed_each(g, u, r, v, n, lane, left);
         }
         if (__any_sync(0xffffffffu, left)) {
@@ -1035,9 +1069,14 @@ extern "C" mhr_status mhr_edge_scores(const mhr_graph* g, const uint32_t* src, c
         MHR_CUDA_TRY(launch_edge_w32(g->dg, ds, dr, dd, n, static_cast<float*>(dout), nullptr, nullptr, nullptr,
                                      nullptr, sms, st));
     } else {
-        if (g->dg.d >= kEdge64Warp)
-            k_edge_scores64_warp<<<sms * 6, kEdge64Warps * 32, 0, st>>>(g->dg, ds, dr, dd, n, static_cast<double*>(dout));
-        else
+        if (g->dg.d >= kEdge64Warp) {
+            const int64_t wave = int64_t(sms) * 6;
+            int per = 32;
+            while (per > 4 && (n + per - 1) / per < wave * kEdge64Warps) per >>= 1;
+            const int64_t blocks = std::min<int64_t>(wave, ((n + per - 1) / per + kEdge64Warps - 1) / kEdge64Warps);
+            k_edge_scores64_warp<<<static_cast<unsigned>(blocks), kEdge64Warps * 32, 0, st>>>(g->dg, ds, dr, dd, n, per,
+                                                                                             static_cast<double*>(dout));
+        } else
             k_edge_scores64<<<sms * 16, 128, 0, st>>>(g->dg, ds, dr, dd, n, static_cast<double*>(dout));
     }
     MHR_CUDA_TRY(cudaGetLastError());

@@ -81,8 +81,10 @@ __device__ __forceinline__ int64_t warp_rows_from(const int64_t* __restrict__ of
 // (3.31 ms; eight rounds at two blocks per SM 3.88 ms; two rounds at four
 // blocks 3.32 ms).
 constexpr int kScoreRounds = 4;
-template <int G, bool SPLIT = false>
-__device__ __forceinline__ float warp_score_v(const DevGraph& g, uint32_t fixv, uint32_t rndv, uint32_t rsa, int lane) {
+// FEW: only the edges of lanes 0 .. n-1 are wanted, n a multiple of the edges of a batch.
+template <int G, bool SPLIT = false, bool FEW = false>
+__device__ __forceinline__ float warp_score_v(const DevGraph& g, uint32_t fixv, uint32_t rndv, uint32_t rsa, int lane,
+                                              int n = 32) {
     constexpr int H = 32 / G;
     constexpr int RB = G < kScoreRounds ? G : kScoreRounds;  // rounds loaded and reduced together
     const unsigned FULL = 0xffffffffu;
@@ -97,6 +99,7 @@ __device__ __forceinline__ float warp_score_v(const DevGraph& g, uint32_t fixv, 
     float wmine = 0.f;
 #pragma unroll
     for (int rb = 0; rb < G; rb += RB) {
+        if (FEW && rb * H >= n) break;
         uint4 C0[RB], C1[RB];
 #pragma unroll
         for (int i = 0; i < RB; ++i) {

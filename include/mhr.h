@@ -164,8 +164,9 @@ typedef struct {
                             all others the threshold search */
     int32_t precision;   /* middle-edge screen: 0 fp32 CUDA cores; 1 bf16 tensor-core
                             contraction with hi/lo split and fp32 accumulation (DistMult,
-                            at most 16 relations); the fp64 rescoring keeps results exact */
-    const mhr_mlp* mlp;  /* order == 2 only */
+                            at most 16 relations); the fp64 rescoring keeps results exact.
+                            The threshold search reads stored fp32 weights with either */
+    const mhr_mlp* mlp;  /* order == 2 only; read by the join */
     int32_t tile;        /* 32-edge groups each warp of the middle join scans per step:
                             0 = default (4), else 4 or 8 (MHR_EINVAL otherwise) */
     int32_t part_count;  /* vertex partition of the paths (the multi-GPU form of Sec. 3.3's
@@ -316,7 +317,9 @@ mhr_status mhr_merge_paths(int32_t nq, int32_t K, int32_t n_parts, const mhr_pat
  * [(p * n_chunks + i) * n_tiles + j], p indexing the screens tried in the
  * order above; *best_chunk, *best_tile and *best_precision (optional) (host)
  * = the fastest combination (the first one on ties).  Every run computes the
- * same result (discarded).  Keeps the winner's buffers and releases the
+ * same result (discarded).  The three shape the join, so on a graph with a
+ * weight index it is the join that is timed (the form of calls with stats and
+ * prune 0 or order 0, and of queries handed back by the threshold search).  Keeps the winner's buffers and releases the
  * others'.  Synchronous.  MHR_EINVAL on bad arguments or candidates.
  */
 mhr_status mhr_autotune(const mhr_graph* g, int32_t nq, const uint32_t* s, const uint32_t* t, int32_t K,

@@ -3057,9 +3057,17 @@ static mhr_status get_plan(mhr_graph* G, int nq, int K, int chunk, int precision
     return MHR_OK;
 }
 
+// what a call wants of a batch besides its lists
+enum class Want {
+    kLists,
+    kCounters,  // the work counters
+    kJoin,      // the join, whatever could answer
+    kLabels     // the join's training labels
+};
+
 static mhr_status run_batch(mhr_graph* G, int nq, const uint32_t* hS, const uint32_t* hT, int K,
-                            const mhr_query_opts* opts, cudaStream_t st, Plan** plan_out, bool counters,
-                            bool label = false) {
+                            const mhr_query_opts* opts, cudaStream_t st, Plan** plan_out, Want want) {
+    const bool label = want == Want::kLabels;
     int chunk = (opts && opts->chunk > 0) ? opts->chunk : kDefaultChunk;
     if (chunk > kMaxChunk || chunk < 32 || (chunk & 31))
         return fail(MHR_EINVAL, "opts->chunk must be a multiple of 32 in [32, 32768]");
@@ -3124,9 +3132,10 @@ static mhr_status run_batch(mhr_graph* G, int nq, const uint32_t* hS, const uint
         p->h.mlp.b2 = m->b2;
     }
     // The threshold search answers every call on a graph with a weight index,
-    // except label runs and those that ask for the counters of a full enumeration
-    // or of the natural order (stats with prune 0 or order 0).
-    const bool searched = G->dg.w && !label && (!counters || (p->h.prune && p->h.order));
+    // except label runs, the autotuner's, and those that ask for the counters of a full
+    // enumeration or of the natural order (stats with prune 0 or order 0).
+    const bool searched =
+        G->dg.w && (want == Want::kLists || (want == Want::kCounters && p->h.prune && p->h.order));
     p->h.label = label ? 1 : 0;
     if (label && (p->h.prune || p->h.order)) return fail(MHR_EINVAL, "label runs use the plain search");
     // vertex partition of the paths by their hop-1 vertex
@@ -3246,7 +3255,7 @@ extern "C" mhr_status mhr_topk_paths_batched(const mhr_graph* gc, int32_t nq, co
         pt = ht.data();
     }
     Plan* p = nullptr;
-    MHR_TRY(run_batch(G, nq, ps, pt, K, opts, st, &p, stats != nullptr));
+    MHR_TRY(run_batch(G, nq, ps, pt, K, opts, st, &p, stats ? Want::kCounters : Want::kLists));
     const cudaMemcpyKind kind = mem == MHR_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     MHR_CUDA_TRY(cudaMemcpyAsync(out, p->h.out, sizeof(mhr_path) * static_cast<size_t>(nq) * K, kind, st));
     MHR_CUDA_TRY(cudaMemcpyAsync(n_out, p->h.n_out, sizeof(int32_t) * nq, kind, st));
@@ -3261,7 +3270,8 @@ extern "C" mhr_status mhr_topk_paths_batched(const mhr_graph* gc, int32_t nq, co
 // Autotuner of the join's launch shape and middle-edge screen: every
 // (screen, work-item size, scan tile) candidate runs the same batch (results
 // do not depend on any of them), timed by the plan's own events; the plans of
-// the losing candidates are released.
+// the losing candidates are released.  It is the join that runs also on a graph with
+// a weight index, whose threshold search reads none of the three.
 extern "C" mhr_status mhr_autotune(const mhr_graph* gc, int32_t nq, const uint32_t* s, const uint32_t* t, int32_t K,
                                    mhr_mem mem, const mhr_query_opts* opts, const int32_t* chunks, int32_t n_chunks,
                                    const int32_t* tiles, int32_t n_tiles, int32_t reps, int32_t* best_chunk,
@@ -3313,10 +3323,10 @@ extern "C" mhr_status mhr_autotune(const mhr_graph* gc, int32_t nq, const uint32
         o.chunk = chunks[(i % per) / n_tiles];
         o.tile = tiles[i % n_tiles];
         Plan* p = nullptr;
-        MHR_TRY(run_batch(G, nq, hs.data(), ht.data(), K, &o, st, &p, false));  // warm-up (capture, buffers)
+        MHR_TRY(run_batch(G, nq, hs.data(), ht.data(), K, &o, st, &p, Want::kJoin));  // warm-up (capture, buffers)
         float ms = 0.f;
         for (int r = 0; r < reps; ++r) {
-            MHR_TRY(run_batch(G, nq, hs.data(), ht.data(), K, &o, st, &p, false));
+            MHR_TRY(run_batch(G, nq, hs.data(), ht.data(), K, &o, st, &p, Want::kJoin));
             mhr_stats sts{};
             MHR_TRY(read_stats(p, st, &sts));
             if (sts.ms_device < 0) return fail(MHR_ECUDA, "autotune: event timing failed");
@@ -3356,7 +3366,7 @@ extern "C" mhr_status mhr_training_labels(const mhr_graph* gc, int32_t nq, const
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     Plan* p = nullptr;
     mhr_query_opts plain{};
-    MHR_TRY(run_batch(G, nq, s, t, 1, &plain, st, &p, true, true));
+    MHR_TRY(run_batch(G, nq, s, t, 1, &plain, st, &p, Want::kLabels));
     unsigned long long* cnt = p->h.counters + kCntLabels;
     MHR_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
     k_dump_labels<<<std::max(1, G->num_sms) * 4, 256, 0, st>>>(reinterpret_cast<const PlanDev*>(p->dregion), cap,

@@ -2682,6 +2682,20 @@ static mhr_status ensure_slots(Plan* p, int64_t X) {
     return MHR_OK;
 }
 
+// Buffers of the threshold search past its blocks' shared memory (376 KB a block, 115 MB
+// for a full GPU), on the first call that runs it.  False when there is no room: the
+// join answers then.
+static bool ensure_spill(Plan* p) {
+    if (p->h.spill_queue) return true;
+    const size_t grid = static_cast<size_t>(p->search_grid);
+    if ((!p->h.spill && plan_alloc(p, &p->h.spill, grid * kSrSpill) != MHR_OK) ||
+        plan_alloc(p, &p->h.spill_queue, grid * kSrSpillQueue) != MHR_OK) {
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
 // The sequence is captured as three graphs (before, the join, after) so that
 // timing events recorded between their launches on the caller's stream bracket
 // the join kernel exactly.
@@ -2963,9 +2977,6 @@ static mhr_status make_plan(mhr_graph* G, int nq, int K, int chunk, int precisio
         // 1,024-thread block per query shortens its phases
         p->search_threads = nq > p->grid ? 512 : 1024;
         p->search_grid = std::min(nq, p->search_threads == 512 ? 2 * p->grid : p->grid);
-        if ((rc = plan_alloc(p, &h.spill, static_cast<size_t>(p->search_grid) * kSrSpill)) != MHR_OK) return bail(rc);
-        if ((rc = plan_alloc(p, &h.spill_queue, static_cast<size_t>(p->search_grid) * kSrSpillQueue)) != MHR_OK)
-            return bail(rc);
     }
     if ((rc = plan_alloc(p, &h.partials, kScanPartials)) != MHR_OK) return bail(rc);
     if (cudaMemset(h.partials, 0, sizeof(int64_t) * kScanPartials) != cudaSuccess)
@@ -3131,11 +3142,13 @@ static mhr_status run_batch(mhr_graph* G, int nq, const uint32_t* hS, const uint
         p->h.mlp.w2 = m->w2;
         p->h.mlp.b2 = m->b2;
     }
-    // The threshold search answers every call on a graph with a weight index,
-    // except label runs, the autotuner's, and those that ask for the counters of a full
-    // enumeration or of the natural order (stats with prune 0 or order 0).
-    const bool searched =
-        G->dg.w && (want == Want::kLists || (want == Want::kCounters && p->h.prune && p->h.order));
+    // The threshold search answers every call on a graph with a weight index (and room
+    // for its buffers), except label runs, the autotuner's, and those that ask for the
+    // counters of a full enumeration or of the natural order (stats with prune 0 or
+    // order 0).
+    const bool searched = G->dg.w &&
+                          (want == Want::kLists || (want == Want::kCounters && p->h.prune && p->h.order)) &&
+                          ensure_spill(p);
     p->h.label = label ? 1 : 0;
     if (label && (p->h.prune || p->h.order)) return fail(MHR_EINVAL, "label runs use the plain search");
     // vertex partition of the paths by their hop-1 vertex

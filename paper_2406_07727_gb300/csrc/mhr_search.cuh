@@ -937,7 +937,8 @@ __device__ void search_query(const DevGraph& g, unsigned long long heavy, unsign
             return;
         }
         // side and probes
-        float last = INFINITY;
+        float last = INFINITY, cut = cutf;
+        int cut_side = fsd;
         for (int trial = 0; trial < 4 && sm.thr_key; ++trial) {
             float level, level1;
             float n = sr_estimate<NT>(&level);
@@ -952,7 +953,11 @@ __device__ void search_query(const DevGraph& g, unsigned long long heavy, unsign
             if (n <= static_cast<float>(kSrProbe) || n <= 4.f * static_cast<float>(spent) || n > 0.6f * last) break;
             last = n;
             const float before = sm.thr_keep;
-            sr_build_far<NT>(cutf);
+            if (sm.fwd != cut_side) {  // the other row is the far one now
+                cut_side = sm.fwd;
+                cut = sm.side[cut_side].n > kSrHashMax ? sr_cut<NT>(cut_side, kSrHashMax * 3 / 4) : neg_inf();
+            }
+            sr_build_far<NT>(cut);
             if (threadIdx.x == 0) sm.cand_cnt = 0;
             __syncthreads();
             spent = sr_scan<NT, false>(true, 0u, level, static_cast<unsigned long long>(n * 0.25f));

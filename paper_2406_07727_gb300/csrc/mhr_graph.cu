@@ -749,14 +749,27 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
     MHR_CUDA_TRY(cudaStreamSynchronize(st));
     if (herr[kErrOffsets])
         return fail(MHR_EINVAL, "offsets must start at 0, be non-decreasing and end at n_edges");
-    // scratch of the reverse sort, and the source of every edge
-    uint32_t* src = nullptr;
+    // scratch, one allocation (for a small graph they are a good part of the load): the
+    // norms' maxima, scan lengths and sums, in-degrees; the reverse sort, and the source
+    // of every edge
+    uint32_t *src = nullptr, *indeg;
+    unsigned long long* mx;  // four maxima in fp64, then the four of the first pass in fp32
+    int64_t *n_dev, *partials;
     SortScratch ss{};
+    const size_t tiles = sort_tiles(static_cast<uint64_t>(E)), nc = 256 * tiles;
+    const size_t eb = (sizeof(uint32_t) * E + 255) / 256 * 256, cb = (sizeof(int64_t) * (nc + 1) + 255) / 256 * 256;
+    const size_t pb = (sizeof(int64_t) * kScanPartials + 255) / 256 * 256, nb = (sizeof(uint32_t) * n + 255) / 256 * 256;
+    char* mem;
+    MHR_CUDA_TRY(tmp.alloc(&mem, 3 * 256 + pb + nb + (E ? 5 * eb + 2 * cb : 0)));
+    mx = reinterpret_cast<unsigned long long*>(mem);
+    n_dev = reinterpret_cast<int64_t*>(mem + 256);
+    ss.n_counts = reinterpret_cast<int64_t*>(mem + 512);
+    ss.partials = partials = reinterpret_cast<int64_t*>(mem + 768);  // left zero by every scan
+    indeg = reinterpret_cast<uint32_t*>(mem + 768 + pb);
+    mem += 768 + pb + nb;
+    MHR_CUDA_TRY(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * 6, st));
+    MHR_CUDA_TRY(cudaMemsetAsync(partials, 0, pb + nb, st));  // and the in-degrees
     if (E) {
-        const size_t tiles = sort_tiles(static_cast<uint64_t>(E)), nc = 256 * tiles;
-        const size_t eb = (sizeof(uint32_t) * E + 255) / 256 * 256, cb = (sizeof(int64_t) * (nc + 1) + 255) / 256 * 256;
-        char* mem;
-        MHR_CUDA_TRY(tmp.alloc(&mem, 5 * eb + 2 * cb + 256 + sizeof(int64_t) * kScanPartials));
         src = reinterpret_cast<uint32_t*>(mem);
         for (int i = 0; i < 2; ++i) {
             ss.key[i] = reinterpret_cast<uint32_t*>(mem + (1 + i) * eb);
@@ -765,11 +778,8 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
         mem += 5 * eb;
         ss.counts = reinterpret_cast<uint32_t*>(mem);
         ss.offsets = reinterpret_cast<int64_t*>(mem + cb);
-        ss.n_counts = reinterpret_cast<int64_t*>(mem + 2 * cb);
-        ss.partials = reinterpret_cast<int64_t*>(mem + 2 * cb + 256);
         const int64_t nch = static_cast<int64_t>(nc);
         MHR_CUDA_TRY(cudaMemcpyAsync(ss.n_counts, &nch, sizeof nch, cudaMemcpyHostToDevice, st));
-        MHR_CUDA_TRY(cudaMemsetAsync(ss.partials, 0, sizeof(int64_t) * kScanPartials, st));
         k_validate_edges<<<grid, 256, 0, st>>>(off, col, rel, n, E, R, src, err);
     }
     k_validate_finite<<<grid, 256, 0, st>>>(vemb, desc->emb_dtype, n * d, err);
@@ -829,13 +839,6 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
     MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&rcol), sizeof(uint32_t) * E));
     MHR_TRY(graph_alloc(g, reinterpret_cast<void**>(&rrel), sizeof(uint16_t) * E));
     {
-        uint32_t* indeg;
-        int64_t *n_dev, *partials;
-        MHR_CUDA_TRY(tmp.alloc(&indeg, sizeof(uint32_t) * n));
-        MHR_CUDA_TRY(tmp.alloc(&n_dev, sizeof(int64_t)));
-        MHR_CUDA_TRY(tmp.alloc(&partials, sizeof(int64_t) * kScanPartials));
-        MHR_CUDA_TRY(cudaMemsetAsync(partials, 0, sizeof(int64_t) * kScanPartials, st));
-        MHR_CUDA_TRY(cudaMemsetAsync(indeg, 0, sizeof(uint32_t) * n, st));
         MHR_CUDA_TRY(cudaMemcpyAsync(n_dev, &n, sizeof(int64_t), cudaMemcpyHostToDevice, st));
         if (E) k_count_in<<<grid, 256, 0, st>>>(col, E, indeg);
         MHR_CUDA_TRY(device_excl_scan<uint32_t>(indeg, n_dev, partials, roff, st));
@@ -879,9 +882,6 @@ mhr_status load_impl(const mhr_graph_desc* desc, mhr_graph* g, cudaStream_t st) 
     MHR_CUDA_TRY(cudaMemcpyAsync(g->h_roff.data(), roff, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, st));
 
     // --- norms
-    unsigned long long* mx;  // four maxima in fp64, then the four of the first pass in fp32
-    MHR_CUDA_TRY(tmp.alloc(&mx, sizeof(unsigned long long) * 6));
-    MHR_CUDA_TRY(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * 6, st));
     unsigned* top = reinterpret_cast<unsigned*>(mx + 4);
     float2* sums = reinterpret_cast<float2*>(src);  // the sort is done with its scratch
     const int64_t most = std::max<int64_t>(n, R);

@@ -48,10 +48,13 @@ static __global__ void __launch_bounds__(kSortThreads)
         counts[static_cast<uint64_t>(d) * tiles + blockIdx.x] = hist[d];
 }
 
-// vals_in == NULL: value i is i; keys_out == NULL: only the values are written
+// vals_in == NULL: value i is i; keys_out == NULL: only the values are written;
+// offsets == NULL: few tiles, whose counts every block adds up itself (none needed
+// for a single tile)
 static __global__ void __launch_bounds__(kSortThreads)
     k_sort_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, uint32_t n, int shift,
-                   uint32_t tiles, const int64_t* __restrict__ offsets, uint32_t* __restrict__ keys_out,
+                   uint32_t tiles, const int64_t* __restrict__ offsets, const uint32_t* __restrict__ counts,
+                   uint32_t* __restrict__ keys_out,
                    uint32_t* __restrict__ vals_out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem& sm = *reinterpret_cast<SortSmem*>(smem_raw);
@@ -90,10 +93,24 @@ static __global__ void __launch_bounds__(kSortThreads)
         }
     }
     const uint32_t lb = block_excl_scan<uint32_t>(tot, sm.red, nullptr);
-    if (threadIdx.x < 256) {
-        sm.lbase[threadIdx.x] = lb;
-        sm.gbase[threadIdx.x] = static_cast<uint32_t>(offsets[static_cast<uint64_t>(threadIdx.x) * tiles + blockIdx.x]) - lb;
+    if (offsets) {
+        if (threadIdx.x < 256)
+            sm.gbase[threadIdx.x] =
+                static_cast<uint32_t>(offsets[static_cast<uint64_t>(threadIdx.x) * tiles + blockIdx.x]) - lb;
+    } else if (tiles == 1) {
+        if (threadIdx.x < 256) sm.gbase[threadIdx.x] = 0u;
+    } else {  // block-uniform
+        uint32_t all = 0u, before = 0u;
+        if (threadIdx.x < 256)
+            for (uint32_t t = 0; t < tiles; ++t) {
+                const uint32_t c = counts[threadIdx.x * tiles + t];
+                all += c;
+                if (t < blockIdx.x) before += c;
+            }
+        const uint32_t first = block_excl_scan<uint32_t>(all, sm.red, nullptr);
+        if (threadIdx.x < 256) sm.gbase[threadIdx.x] = first + before - lb;
     }
+    if (threadIdx.x < 256) sm.lbase[threadIdx.x] = lb;
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kSortItems; ++j) {
@@ -123,6 +140,11 @@ struct SortScratch {
     int64_t* partials;  // kScanPartials, zero
 };
 
+// Up to this many tiles (131,072 pairs) a pass needs no scan of the counts, and one
+// tile no counts: one or two launches instead of four, of about 3 us each when there is
+// next to nothing to sort.
+constexpr uint32_t kSortFewTiles = 16;
+
 inline uint32_t sort_tiles(uint64_t n) { return static_cast<uint32_t>((n + kSortTile - 1) / kSortTile); }
 
 // Sorts the pairs (keys[i], vals[i]) (vals == NULL: (keys[i], i)) by the low
@@ -137,10 +159,14 @@ inline cudaError_t radix_sort_pairs(const uint32_t* keys, const uint32_t* vals, 
     int side = vals == s.val[0] || keys == s.key[0] ? 1 : 0;  // never in place
     for (int shift = 0; shift < bits || shift == 0; shift += 8) {
         const bool last = shift + 8 >= bits;
-        k_sort_count<<<tiles, kSortThreads, 0, st>>>(keys, n, shift, tiles, s.counts);
-        e = device_excl_scan<uint32_t>(s.counts, s.n_counts, s.partials, s.offsets, st);
-        if (e != cudaSuccess) return e;
-        k_sort_scatter<<<tiles, kSortThreads, sizeof(SortSmem), st>>>(keys, vals, n, shift, tiles, s.offsets,
+        const bool few = tiles <= kSortFewTiles;
+        if (tiles > 1) k_sort_count<<<tiles, kSortThreads, 0, st>>>(keys, n, shift, tiles, s.counts);
+        if (!few) {
+            e = device_excl_scan<uint32_t>(s.counts, s.n_counts, s.partials, s.offsets, st);
+            if (e != cudaSuccess) return e;
+        }
+        k_sort_scatter<<<tiles, kSortThreads, sizeof(SortSmem), st>>>(keys, vals, n, shift, tiles,
+                                                                      few ? nullptr : s.offsets, s.counts,
                                                                       last ? nullptr : s.key[side], s.val[side]);
         keys = s.key[side];
         vals = s.val[side];

@@ -18,8 +18,9 @@ Output: one JSON line on rank 0.
   e2e         the same metric through the C ABI with host buffers: host->device
               copy of the queries and device->host copy of the results inside
               the timed region (wall clock)
-  roofline    middle-join kernel: algorithmic bytes / its event-timed duration
-              against the measured HBM copy bandwidth
+  roofline    threshold search (graphs with a weight index) or middle join:
+              algorithmic bytes / its event-timed duration against the measured
+              HBM copy bandwidth
   cpu_baseline the CPU oracle (fp64 brute force, OpenMP over queries) on a
               bounded sample of the same queries
   oracle_parity every query of that sample compared with the GPU result
@@ -83,15 +84,17 @@ WORKLOAD_DESCS = {
 K_OVERRIDE = 0
 WORKLOAD_DESC = WORKLOAD_DESCS[WORKLOAD]
 DATA = "synthetic: seeded R-MAT typed knowledge graph standing in for WikiKG90Mv2"
-FORM_DESC = {"plain": "plain: batched, threshold search over the weight index (every middle edge scored when the "
-                      "graph has none), fp32 screen + fp64 rescoring",
+# on a graph with a weight index every form is the same search (identical lists)
+SEARCH_DESC = ("threshold search over the weight index (fp32 screen + fp64 rescoring): it reads edges by their stored "
+               "weights, so the form's row order, pruning and learned scores are not used")
+FORM_DESC = {"plain": "plain: batched join, every middle edge scored, fp32 screen + fp64 rescoring",
              "bound": "bound: plain + rows ordered by their score bound, a seed pass per query, provable "
                       "bound pruning of work items, rows and hits (identical output)",
              "chosen": "chosen: as bound, with rows ordered by the learned MLP score (trained on plain runs "
                        "over 20,000 held-out queries before timing) (identical output)"}
-# kernels per step of the threshold search (graphs with a weight index): k_init, k_search, k_rescore,
+# kernels per step of the threshold search (graphs with a weight index): k_search, k_rescore,
 # k_merge2; queries it hands back run the join below in a conditional node
-SEARCH_KERNELS_PER_STEP = 4
+SEARCH_KERNELS_PER_STEP = 3
 # kernels per step of the join: k_init, k_expand_v, scan x2, k_lists, k_plan, k_order_key, k_mlp_qbias,
 # k_mlp_keys, k_order_hist, scan x2, k_order_perm, scan x2, k_near, k_middle (seed),
 # k_middle, k_merge1, k_rescore, k_merge2, k_exact
@@ -151,6 +154,13 @@ def close_replicas(ws: int):
 def job_rate(units_per_rank: int, ws: int, steps: int, max_ms: float) -> float:
     """Whole-job throughput: units all ranks processed / the slowest rank's time."""
     return units_per_rank * ws * steps / (max_ms / 1000.0)
+
+
+def has_index(mhr, G, s, t) -> bool:
+    """Whether the graph has a weight index: the expansion, a part of the join only, then has no time of its own."""
+    st = mhr.mhr_topk_paths_batched(G, np.array([s], np.uint32), np.array([t], np.uint32), 1,
+                                    opts={"prune": 1, "order": 1}, with_stats=True)[2]
+    return st["ms_expand"] == 0.0
 
 
 def load_workload(rank: int):
@@ -540,7 +550,8 @@ BEAM_METRIC = "beam-search queries/s (Alg. 6 / Alg. 7, H=3, K=10) on 1 GB300, re
 def run_beam(args):
     """Beam search: CUDA events around each call (queries as host arrays of
     512 B, results copied back inside the call), L2 flushed before every call;
-    roofline of the edge scoring against the fp32 add rate."""
+    roofline of the rows read (with a weight index) or of the edge scoring
+    against the fp32 add rate (without)."""
     import torch
     import synth
     import paper_2406_07727_gb300 as mhr
@@ -552,6 +563,7 @@ def run_beam(args):
     g, S, T, _, _ = synth.workload("medium")
     S, T = rank_queries(g, S, T, rank, "medium")
     G = mhr.load_kg(g)
+    indexed = has_index(mhr, G, S[0], T[0])
     stream = torch.cuda.current_stream()
     flush = torch.empty(256 * 1024 * 1024, dtype=torch.uint8, device="cuda")
     for _ in range(args.warmup):
@@ -572,14 +584,30 @@ def run_beam(args):
     value = job_rate(len(S), ws, args.steps, tot_ms)
     if rank == 0:
         ms = tot_ms / args.steps
-        # TransE-L1: an add, a subtract and an accumulate per element of every
-        # out-edge of every held path (screened in fp32; the band near each
-        # path's K-th extension rescored in fp64)
-        flops = 3.0 * g.d * st["edges_scanned"]
-        achieved = flops / (ms / 1000.0) / 1e12
-        n_sms = torch.cuda.get_device_properties(0).multi_processor_count
-        sm_mhz = (clk or {}).get("sm_mhz") or 2070.0
-        alu_peak = n_sms * 128 * sm_mhz * 1e6 / 1e12
+        eb = 4 if g.dtype == "f32" else 2
+        if indexed:
+            # a warp per held path reads the front of its sorted row (10 B an edge) and the rows of the edges it
+            # scores in fp64; the rest of the row is not touched
+            moved = st["rescored"] * (10 + eb * g.d)
+            peak, peak_src = measured_peaks()
+            roofline = {"bound": "hbm", "achieved": moved / (ms / 1000.0) / 1e9, "peak": peak, "unit": "GB/s",
+                        "frac": moved / (ms / 1000.0) / 1e9 / peak, "traffic": None,
+                        "kernel": "k_beam_step (all levels of a call)", "peak_source": f"{peak_src} hbm_gbs",
+                        "bytes_per_call": moved,
+                        "note": "a chain of dependent loads per level and the call's launches and waits bound it"}
+        else:
+            # TransE-L1: an add, a subtract and an accumulate per element of every
+            # out-edge of every held path (screened in fp32; the band near each
+            # path's K-th extension rescored in fp64)
+            flops = 3.0 * g.d * st["edges_scanned"]
+            achieved = flops / (ms / 1000.0) / 1e12
+            n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+            sm_mhz = (clk or {}).get("sm_mhz") or 2070.0
+            alu_peak = n_sms * 128 * sm_mhz * 1e6 / 1e12
+            roofline = {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",
+                        "frac": achieved / alu_peak, "traffic": None, "kernel": "k_beam_level (all levels of a call)",
+                        "peak_source": f"{n_sms} SMs x 128 fp32 lanes x {sm_mhz:.0f} MHz (adds)",
+                        "flops_per_call": flops}
         cpu = None
         if ws == 1 and not args.no_cpu:
             import oracle
@@ -604,15 +632,11 @@ def run_beam(args):
                        "call": "mhr_beam_paths, synchronous; host arrays in and out"},
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 8 * len(S),
                     "d2h_bytes_per_step": len(S) * BEAM_K * 64 + 4 * len(S)},
-            "gpu_launches": (2 * BEAM_H + 2) * args.steps,
-            "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",
-                         "frac": achieved / alu_peak, "traffic": None,
-                         "kernel": "k_beam_step / k_beam_level (all levels of a call; every out-edge of a held path "
-                                   "counts, read or not)",
-                         "peak_source": f"{n_sms} SMs x 128 fp32 lanes x {sm_mhz:.0f} MHz (adds)",
-                         "flops_per_call": flops},
+            # the first level's paths, one or two kernels per level, the final order
+            "gpu_launches": ((2 if indexed else 1) * BEAM_H + 2) * args.steps,
+            "roofline": roofline,
             "clocks": clk,
-            "work_per_step": {"edges_scored_fp32": st["edges_scanned"], "edges_rescored_fp64": st["rescored"]},
+            "work_per_step": {"out_edges_of_held_paths": st["edges_scanned"], "edges_rescored_fp64": st["rescored"]},
         }
         if cpu is not None:
             line["cpu_baseline"] = cpu
@@ -639,6 +663,7 @@ def run_gpu(args):
     nq = len(S)
     score_fn = spec.get("score", "transe")
     G = mhr.load_kg(g, score_fn=score_fn)
+    searched = has_index(mhr, G, S[0], T[0])
     tc = 1 if score_fn == "distmult" else 0   # tensor-core middle-edge screen for DistMult
     stream = torch.cuda.current_stream()
     dS = torch.from_numpy(S.astype(np.int32)).cuda()
@@ -648,7 +673,7 @@ def run_gpu(args):
     flush = torch.empty(256 * 1024 * 1024, dtype=torch.uint8, device="cuda")  # > 129 MB L2
 
     model, train_rep, train_s = None, None, 0.0
-    if args.form == "chosen" or args.all_forms:
+    if not searched and (args.form == "chosen" or args.all_forms):
         t0 = time.perf_counter()
         import synth
         # training queries: the workload's own recipe on stream 3 (disjoint from the timed ones)
@@ -667,14 +692,16 @@ def run_gpu(args):
             o = {"prune": 0, "order": 0}
         elif form == "bound":
             o = {"prune": 1, "order": 1, "precision": tc}
+        elif searched:  # no order of the rows is read, so there is none to learn
+            o = {"prune": 1, "order": 1, "precision": tc}
         else:
             o = {"prune": 1, "order": 2, "mlp": model, "precision": tc}
         if args.chunk > 0:
             o["chunk"] = args.chunk
-        elif args.chunk < 0:
+        elif args.chunk < 0 and (not searched or form == "plain"):
             # launch shape (work-item size, scan tile) and, for DistMult, the
             # middle-edge screen from the library's autotuner, on this batch,
-            # before timing
+            # before timing; with an index they shape the plain form's counters only
             if form not in tuned:
                 to = dict(o)
                 if tc and form != "plain":
@@ -749,8 +776,11 @@ def run_gpu(args):
             continue
         o_steps = max(3, args.steps // 4)
         o_ms, o_join, o_dev, o_stats, _ = timed(make_opts(of), o_steps)
-        others[of] = {"form": FORM_DESC[of], "value": job_rate(nq, ws, o_steps, o_ms),
-                      "ms_per_step": o_ms / o_steps, "join_ms": statistics.mean(o_join),
+        others[of] = {"form": SEARCH_DESC if searched else FORM_DESC[of], "value": job_rate(nq, ws, o_steps, o_ms),
+                      "ms_per_step": o_ms / o_steps,
+                      # the plain form's counters need every edge: with an index those calls alone run the join
+                      ("counters_join_ms" if searched and of == "plain" else "search_ms" if searched else "join_ms"):
+                          statistics.mean(o_join),
                       "chunk": tuned[of][0] if of in tuned else args.chunk,
                       "tile": tuned[of][1] if of in tuned else None,
                       "middle_edge_screen": (("bf16 tensor cores" if tuned[of][2] else "fp32 CUDA cores")
@@ -787,9 +817,8 @@ def run_gpu(args):
         alg_bytes = 4 * s_near + 2 * plain_stats["hits"] + eb * g.d * n_vert
         moved_bytes = 4 * stats["edges_scanned"] + 2 * stats["hits"] + eb * g.d * n_vert
         join_avg_ms = statistics.mean(join_ms)
-        # the expansion is a part of the join's graphs only: no time of it, the threshold search ran
-        searched = expand_ms[0] == 0.0
-        if searched:  # 8 B (vertex, weight) per middle edge read, its result written
+        by_search = searched and args.form != "plain"  # whose counters and kernel time these are
+        if by_search:  # 8 B (vertex, weight) per middle edge read, its result written
             moved_bytes = alg_bytes = 8 * stats["edges_scanned"] + 24 * nq * K
         achieved = alg_bytes / (join_avg_ms / 1000.0) / 1e9
         peak, peak_src = measured_peaks()
@@ -804,8 +833,9 @@ def run_gpu(args):
             "warmup": args.warmup, "ms_per_step": elapsed_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32+f64", "data": DATA,
             "config": {"workload": WORKLOAD_DESC, "queries_per_step": nq, "K": K,
-                       "score_fn": score_fn, "form": FORM_DESC[args.form],
-                       "middle_edge_screen": ("bf16 tensor cores (hi/lo split)" if opts.get("precision") == 1
+                       "score_fn": score_fn, "form": SEARCH_DESC if searched else FORM_DESC[args.form],
+                       "middle_edge_screen": ("fp32 weights stored in the index" if searched else
+                                              "bf16 tensor cores (hi/lo split)" if opts.get("precision") == 1
                                               else "fp32 CUDA cores"),
                        "l2": "flushed before every step (256 MiB write, excluded from the step time)",
                        "parallelism": "replicas (each rank its own queries)" if ws > 1 else "single GPU",
@@ -821,14 +851,16 @@ def run_gpu(args):
             "gpu_launches": (SEARCH_KERNELS_PER_STEP if searched else KERNELS_PER_STEP) * args.steps,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak,
-                         "traffic": (None if searched else
+                         "traffic": (None if by_search else
                                      TRAFFIC_NCU.get((WORKLOAD, args.form, opts.get("chunk"), opts.get("tile")))),
                          "traffic_scope": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the main join launch",
-                         "kernel": "k_search (threshold search)" if searched else "k_middle (middle join)", "peak_source": f"{peak_src} hbm_gbs",
+                         "kernel": "k_search (threshold search)" if by_search else "k_middle (middle join)",
+                         "peak_source": f"{peak_src} hbm_gbs",
                          "alg_bytes_per_launch": alg_bytes, "avg_launch_ms": join_avg_ms,
                          "bytes_moved_per_launch": moved_bytes,
-                         "note": ("bytes of the middle edges the search reads (its phases wait on latency); the plain method reads "
-                                  f"{4 * s_near} bytes of them" if searched else
+                         "note": ("bytes of the middle edges the search reads (its phases wait on latency); the plain "
+                                  "method reads "
+                                  f"{4 * s_near} bytes of them" if by_search else
                                   "achieved credits the plain method's algorithmic bytes (effective rate for the pruned form)")},
             "clocks": clk,
             "scored_paths_per_s": paths_per_s,
@@ -848,7 +880,8 @@ def run_gpu(args):
             "join_ms_spread": {"min": min(join_ms), "median": statistics.median(join_ms), "max": max(join_ms)},
             "steps_with_dense_queries": sum(1 for x in dense_steps if x),
             "stats_steps": "work counters, device/join times and dense counts come from up to 10 untimed "
-                           "steps of the same work after the timed loop",
+                           "steps after the timed loop, of the same work except the plain form's on a graph with "
+                           "an index: its counters are the join's, which enumerates every middle edge",
             "device_host_agree": agree,
             "wall_s_timed_loop": wall1 - wall0,
         }
@@ -861,7 +894,7 @@ def run_gpu(args):
         slots = sum(f["deg_s"] + f["deg_t"] for f in fs)
         x_bytes = slots * (4 + 2) + eb * g.d * (n_vert + 2 * nq)
         x_ms = expand_ms[0]
-        result["expansion_roofline"] = None if searched else {
+        result["expansion_roofline"] = None if x_ms == 0.0 else {
             "bound": "hbm", "kernel": "k_expand (hop-1 / hop-3 expansion)",
             "achieved": x_bytes / (x_ms / 1000.0) / 1e9, "peak": peak, "unit": "GB/s",
             "frac": x_bytes / (x_ms / 1000.0) / 1e9 / peak, "alg_bytes_per_launch": x_bytes,

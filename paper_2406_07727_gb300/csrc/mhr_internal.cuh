@@ -63,7 +63,8 @@ struct DevGraph {
     const float* maxw_out;
     const float* maxw_in;
     // the same per (vertex, relation): [n x R], entry v * R + r; NULL when
-    // n x R exceeds kMaxRelBoundEntries
+    // n x R exceeds kMaxRelBoundEntries and, with the weight index, until a
+    // pruned join first asks for them (build_rel_bounds)
     const float* maxw_out_r;
     const float* maxw_in_r;
     // weight index (all NULL when the graph has none): the fp32 weight of every
@@ -114,6 +115,7 @@ struct mhr_graph {
     // per-edge bound and the path bound when w2 comes from it
     double epstc_edge = 0, err_path_tc = 0;
     uint16_t* wsplit = nullptr;  // [2][R][d] bf16 hi / lo parts of the relation table
+    bool rel_bounds_tried = false;
     double max_l1 = 0, max_rel_l1 = 0, max_rel_inf = 0, max_l2sq = 0;
     int num_sms = 0;
     mhr::PlanCache* plans = nullptr;
@@ -270,5 +272,7 @@ __host__ __device__ inline int score_group_width(int d, int dtype) {
 // host helpers
 int device_sm_count();
 mhr_status check_graph(const mhr_graph* g);
+// per (vertex, relation) bounds of a graph with a weight index, if they fit
+void build_rel_bounds(mhr_graph* g, cudaStream_t st);
 
 }  // namespace mhr

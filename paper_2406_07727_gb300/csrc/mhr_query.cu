@@ -2537,12 +2537,15 @@ struct Plan {
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // before / join / after / end
     cudaEvent_t ev_x[2] = {nullptr, nullptr};  // around the expansion kernel (recorded inside the first graph)
     bool h2d_pending = false;
-    void drop_graphs() {
+    void drop_join_graphs() {
         for (cudaGraphExec_t& x : exec)
             if (x) {
                 cudaGraphExecDestroy(x);
                 x = nullptr;
             }
+    }
+    void drop_graphs() {
+        drop_join_graphs();
         if (exec_search) cudaGraphExecDestroy(exec_search);
         exec_search = nullptr;
     }
@@ -3149,6 +3152,11 @@ static mhr_status run_batch(mhr_graph* G, int nq, const uint32_t* hS, const uint
     const bool searched = G->dg.w &&
                           (want == Want::kLists || (want == Want::kCounters && p->h.prune && p->h.order)) &&
                           ensure_spill(p);
+    if (!searched && p->h.prune && G->dg.w && !G->rel_bounds_tried) {
+        build_rel_bounds(G, st);
+        // captured joins hold the graph's pointers
+        for (auto& kv : G->plans->plans) kv.second->drop_join_graphs();
+    }
     p->h.label = label ? 1 : 0;
     if (label && (p->h.prune || p->h.order)) return fail(MHR_EINVAL, "label runs use the plain search");
     // vertex partition of the paths by their hop-1 vertex

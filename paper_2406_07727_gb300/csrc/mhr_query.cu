@@ -2691,9 +2691,11 @@ static mhr_status ensure_slots(Plan* p, int64_t X) {
 static bool ensure_spill(Plan* p) {
     if (p->h.spill_queue) return true;
     const size_t grid = static_cast<size_t>(p->search_grid);
+    const std::string keep = mhr_last_error();  // the call itself does not fail
     if ((!p->h.spill && plan_alloc(p, &p->h.spill, grid * kSrSpill) != MHR_OK) ||
         plan_alloc(p, &p->h.spill_queue, grid * kSrSpillQueue) != MHR_OK) {
         cudaGetLastError();
+        set_error(keep);
         return false;
     }
     return true;
@@ -3189,7 +3191,7 @@ static mhr_status run_batch(mhr_graph* G, int nq, const uint32_t* hS, const uint
         if (p->h.order == 0) p->h.order = 1;
         p->h.heavy = int64_t(1) << 22;
         // Without a threshold (fewer than K paths found) every middle edge has to be
-        // read.  One block reads 1.7 G edges/s, the join 73 G edges/s after 0.2 ms of
+        // read.  One block reads about 1.2 G edges/s, the join 73 G edges/s after 0.2 ms of
         // launches: a lone query is better off there past 2^18 edges, and a batch keeps
         // its blocks busy for longer.
         p->h.alone = std::min<int64_t>(p->h.heavy, (int64_t(1) << 18) + (int64_t(nq) << 14));

@@ -37,7 +37,11 @@ def test_search_buffers_come_with_the_search():
     before = free()
     hog = torch.empty(before - (48 << 20), dtype=torch.uint8, device="cuda")  # less than either buffer takes
     assert free() < spill
+    with pytest.raises(mhr.MhrError):
+        mhr.mhr_topk_paths(G, 1, 1, 5)
+    said = mhr.mhr_last_error()
     same(*mhr.mhr_topk_paths_batched(G, S, T, 5))
+    assert mhr.mhr_last_error() == said  # no call has failed since
     del hog
     torch.cuda.empty_cache()
     before = free()

@@ -209,8 +209,12 @@ typedef struct {
  * bound and, when it fits, the weight index: the fp32 weight of every edge and
  * both adjacencies with each row sorted by it (36 bytes per edge, 80 per vertex;
  * kept when it takes at most half of the device memory that is free beside the
- * graph, and stays within the memory cap below).  Results do not depend on it.  Validates the description (MHR_EINVAL with a message on any
- * violation).  Synchronous; *out is NULL on failure, and a failed load has
+ * graph, and stays within the memory cap below).  Results do not depend on it;
+ * searches without it take up to thirty times as long (a call with stats, prune 1
+ * and order 1 shows it: ms_expand is 0 with the index).  Without the index, or
+ * when a call asks for the counters of the pruned natural order, bounds per vertex
+ * and relation are kept (8 bytes each, up to 2^29 of them, within the cap).
+ * Validates the description (MHR_EINVAL with a message on any violation).  Synchronous; *out is NULL on failure, and a failed load has
  * released every device allocation it made.  A service that must keep the
  * graph within a memory budget sets the environment variable
  * MHR_GRAPH_MEMORY_CAP_BYTES (decimal bytes, read at every load): a load

@@ -41,25 +41,3 @@ def test_edge_counts_around_the_forms(E, n):
     for q in range(len(S)):
         assert out[q][: n_out[q]].tobytes() == want[q][: n_want[q]].tobytes()
         assert beams["score"][q][: n_beams[q]].tobytes() == want_b["score"][q][: n_want_b[q]].tobytes()
-
-
-def test_a_tiny_load_takes_no_longer_than_its_launches():
-    """20 edges: the load's kernels are some 35 launches and its buffers 20 allocations.  With four launches for each of
-    seven sort passes it took 0.64 ms."""
-    import time
-    import paper_2406_07727_gb300 as mhr
-    import torch
-    rng = np.random.default_rng(0)
-    off, cols, rels = synth.canonicalize(10, 2, rng.integers(0, 10, 20), rng.integers(0, 2, 20), rng.integers(0, 10, 20))
-    a = [torch.from_numpy(x).cuda() for x in (off, cols.astype(np.int32), rels.astype(np.int16),
-                                              rng.standard_normal((10, 4)).astype(np.float32),
-                                              rng.standard_normal((2, 4)).astype(np.float32))]
-    best = 1.0
-    for _ in range(30):
-        torch.cuda.synchronize()
-        t0 = time.perf_counter()
-        G = mhr.mhr_graph_load(*a, 2)
-        best = min(best, time.perf_counter() - t0)
-        G.close()
-    print(best)
-    assert best < 0.45e-3, best
